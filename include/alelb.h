@@ -71,8 +71,9 @@ enum { ALELB_ELEM_P2TRI = 0, ALELB_ELEM_Q2QUAD = 1 };
 enum { ALELB_RENUMBER_NONE = 0, ALELB_RENUMBER_MORTON = 1 };
 /* Storage and arithmetic of a solver (Sec. IV's populations; the paper
    computes in FP64 and gives no reduced-precision form):
-     FP64      full populations and fields in FP64, FP64 arithmetic, every
-               departure point through the exact element walk;
+     FP64      full populations and fields in FP64, FP64 departure points
+               and arithmetic; element decisions certified in FP32 where that
+               is possible, exact otherwise;
      FP32_DEV  populations stored in FP32 as deviations from the rest
                equilibria at (rho_inf, T_inf), fields in FP32, FP32
                arithmetic with FP64 (certified) element decisions;
@@ -278,9 +279,10 @@ alelb_status alelb_kernel_times(alelb_solver *s, const char **names, double *ms,
                                 int64_t *launches, int32_t *n);
 
 /* Sizes and counters: out = {n_nodes, n_elems, bytes per stored population
-   value, 0, n_wall_nodes, precision, n_wall_edges, element walks run by the
-   propagation kernel since lb_init (populations not settled by the verified
-   previous-step element)}.  Synchronous. */
+   value, 0, n_wall_nodes, precision, n_wall_edges, populations since lb_init that
+   the verified previous-step element did not settle (deviation forms), or
+   all that were located (FP64: every population whose c^ is not exactly
+   zero)}.  Synchronous. */
 alelb_status alelb_info(alelb_solver *s, double out[8]);
 
 /* One FP64 time step t -> t + 1 that allocates nothing (the paper has no

@@ -11,6 +11,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <unordered_map>
 #include <vector>
 
@@ -183,6 +184,7 @@ extern "C" alelb_status alelb_mesh_create(const alelb_mesh_desc *d, alelb_mesh *
     D.nscale = B.put(T.nscale, st);
     D.bkind = B.put(T.bkind, st);
     D.vzero = B.put(T.vzero, st);
+    D.nvzero = (int)std::count(T.vzero.begin(), T.vzero.end(), (uint8_t)1);
     D.cone = B.put(T.cone, st);
     D.conek = B.put(T.conek, st);
     D.wall_idx = B.put(T.wall_idx, st);
@@ -191,6 +193,7 @@ extern "C" alelb_status alelb_mesh_create(const alelb_mesh_desc *d, alelb_mesh *
     D.wall_nrm = B.put(T.wall_nrm, st);
     D.orig_elem = B.put(T.orig, st);
     D.ejf = B.put(T.ejf, st);
+    D.ejd = B.put(T.ejd, st);
     D.bdist = B.put(T.bdist, st);
     D.Xf = B.put(T.Xf, st);
     D.v0f = B.put(T.v0f, st);
@@ -490,7 +493,11 @@ cudaError_t launch_step(alelb_solver *s, StateDev<S> &st, KinParams<A> &K, const
         return cudaGetLastError();
     }
     int seq[KT_N], ns = 0;
-    if (fast) {
+    // The two passes in every form; the FP64 form keeps the plain pass where
+    // no FP32 certificate covers the departure point, so that nothing would
+    // settle in the first one.
+    const bool passes = fast || !(s->flags & (ALELB_FLAG_LITERAL_VG | ALELB_FLAG_EXACT_CHAR));
+    if (passes) {
         seq[ns++] = KT_FAST;
         if (s->mlp) seq[ns++] = KT_PROPOSE;
         seq[ns++] = KT_SLOW;
@@ -516,15 +523,35 @@ cudaError_t launch_step(alelb_solver *s, StateDev<S> &st, KinParams<A> &K, const
         case KT_FAST:
             // one thread per node saves the nine map evaluations of a node,
             // which count on large meshes unless the map is a translation
+            if constexpr (std::is_same<S, double>::value) {
+                // Directions per thread of the FP64 form.  A translation has no
+                // per-node FP64 work, so one (16.6 us against 17.9 and 31.1 at
+                // three and nine on 11.8k nodes, equal from 90k on).  Other maps
+                // cost about as much per thread as a population: nine per thread
+                // where the nodes alone fill the FP64 pipes (160k box: 137 us,
+                // 144 at three, 193 at one; 91k pitch: 82, 86, 117), three below
+                // (24k blended: 34 us against 43 at one and 44 at nine), one
+                // where threads are few (1k box: 10, 17, 34; equal at 9k).
+                const dim3 gb(FAST_BS), g1((N + FAST_BS - 1) / FAST_BS, NQ), g3(g1.x, NQ / 3), g9(g1.x, 1);
+                if (m->T.mkind == MK_NONE || m->T.mkind == MK_PLUNGE)
+                    launch_pdl(k_stream_fast<S, A, 1, true>, g1, gb, s->stream, m->dev, m->mst, scd, sfd, K, st);
+                else if (N < FAST64_G3_NODES)
+                    launch_pdl(k_stream_fast<S, A, 1, false>, g1, gb, s->stream, m->dev, m->mst, scd, sfd, K, st);
+                else if (N < FAST64_G9_NODES)
+                    launch_pdl(k_stream_fast<S, A, 3, false>, g3, gb, s->stream, m->dev, m->mst, scd, sfd, K, st);
+                else
+                    launch_pdl(k_stream_fast<S, A, NQ, false>, g9, gb, s->stream, m->dev, m->mst, scd, sfd, K, st);
+                break;
+            }
             if (m->T.mkind == MK_NONE || m->T.mkind == MK_PLUNGE)
                 launch_pdl(k_stream_fast<S, A, FAST_G, true>, dim3((N + FAST_BS - 1) / FAST_BS, NQ / FAST_G),
-                           dim3(FAST_BS), s->stream, m->dev, m->mst, sfd, K, st);
+                           dim3(FAST_BS), s->stream, m->dev, m->mst, scd, sfd, K, st);
             else if (N < FAST_G_NODES)
                 launch_pdl(k_stream_fast<S, A, FAST_G, false>, dim3((N + FAST_BS - 1) / FAST_BS, NQ / FAST_G),
-                           dim3(FAST_BS), s->stream, m->dev, m->mst, sfd, K, st);
+                           dim3(FAST_BS), s->stream, m->dev, m->mst, scd, sfd, K, st);
             else
                 launch_pdl(k_stream_fast<S, A, NQ, false>, dim3((N + FAST_BS - 1) / FAST_BS, 1), dim3(FAST_BS),
-                           s->stream, m->dev, m->mst, sfd, K, st);
+                           s->stream, m->dev, m->mst, scd, sfd, K, st);
             break;
         case KT_SLOW: {
             // every block resident at once: the list is spread over all

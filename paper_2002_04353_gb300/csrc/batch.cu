@@ -90,35 +90,21 @@ template <class S, class A> struct SharedCase {
     }
 };
 
-template <class S, class A>
-__global__ void __launch_bounds__(256) kb_stream(const CaseDev<S, A> *__restrict__ cases,
-                                                 const int *__restrict__ off, int B,
-                                                 const MapScalars *__restrict__ sc, int count)
-{
-    wait_prior_grid();
-    __shared__ SharedCase<S, A> sh;
-    const int c = tile_case(off, B, blockIdx.x);
-    sh.load(cases, sc, nullptr, c);
-    __syncthreads();
-    const CaseDev<S, A> &C = sh.C();
-    const int a = (blockIdx.x - __ldg(off + c)) * blockDim.x + threadIdx.x;
-    if (a < C.M.N) stream_plain_node(C.M, C.MS, sh.SC(), sh.SC(), C.K, C.st, C.err, count ? C.stats : nullptr, a);
-}
-
 // G directions per thread (grid y: 9 / G groups), chosen by the tuner:
 // one map evaluation per thread, fewer and longer load chains as G grows.
 template <class S, class A, int G>
 __global__ void __launch_bounds__(256) kb_fast(const CaseDev<S, A> *__restrict__ cases,
                                                const int *__restrict__ off, int B,
+                                               const MapScalars *__restrict__ sc,
                                                const MapScalarsF *__restrict__ sf)
 {
     wait_prior_grid();
     __shared__ SharedCase<S, A> sh;
     const int c = tile_case(off, B, blockIdx.x);
-    sh.load(cases, nullptr, sf, c);
+    sh.load(cases, std::is_same<S, double>::value ? sc : nullptr, sf, c); // the FP64 form's departure points
     __syncthreads();
     const CaseDev<S, A> &C = sh.C();
-    stream_fast_group<G>(C.M, C.MS, sh.SF(), C.K, C.st, (blockIdx.x - __ldg(off + c)) * blockDim.x + threadIdx.x);
+    stream_fast_group<G>(C.M, C.MS, sh.SC(), sh.SF(), C.K, C.st, (blockIdx.x - __ldg(off + c)) * blockDim.x + threadIdx.x);
 }
 
 // The exact path over the work lists of all cases as one list, numbered
@@ -160,8 +146,8 @@ __global__ void __launch_bounds__(256) kb_slow(const CaseDev<S, A> *__restrict__
                 run += loc[i];
             }
             if (lane == B - 1) pre[nseg] = run;
-            if (count && npop && blockIdx.x == 0 && cases[lane].stats)
-                atomicAdd(cases[lane].stats, (unsigned long long)npop);
+            if (count && blockIdx.x == 0 && cases[lane].stats)
+                atomicAdd(cases[lane].stats, step_count<S>(cases[lane].M, cases[lane].K.flags, npop));
         }
     }
     __syncthreads();
@@ -177,10 +163,11 @@ __global__ void __launch_bounds__(256) kb_slow(const CaseDev<S, A> *__restrict__
         const CaseDev<S, A> &C = cases[c];
         const int entry = C.st.work[(size_t)i * C.M.N + (w - pre[lo])];
         if (i < NQ) {
-            stream_slow_item(C.M, C.MS, sc[c], sf[c], sc[c], sf[c], C.K, C.st, C.err, entry);
+            const bool own = stream_slow_item(C.M, C.MS, sc[c], sf[c], sc[c], sf[c], C.K, C.st, C.err, entry);
+            if (count) count_own<S>(C.stats, own);
         } else {
             const unsigned mask = C.st.wmask[entry] & WMASK_DIRS;
-            if (count && C.stats) atomicAdd(C.stats, (unsigned long long)__popc(mask));
+            if (count) count_wall<S>(C.stats, mask);
             stream_bc_node<S, A>(C.M, C.MS, sc[c], sf[c], C.K, C.st, entry,
                                  fast_map(C.MS, sf[c], entry, C.M.Xf[entry]), mask);
         }
@@ -600,71 +587,66 @@ __global__ void __launch_bounds__(128) kb_persistent(const CaseDev<S, A> *__rest
     for (int k = 0; k < K; ++k) {
         const MapScalars *sc = scs + (size_t)k * B;
         const MapScalarsF *sf = sfs + (size_t)k * B;
-        if (FAST) {
-            tiles_loop(k, [&](const CaseDev<S, A> &C, const MapScalars &, const MapScalarsF &SF, int a) {
-                stream_fast_group<BATCH_FAST_G>(C.M, C.MS, SF, C.K, C.st, a);
-            });
-            if (!grid_barrier(g, cases, B)) return;
-            // the exact path over every case's work list (kb_slow's numbering)
-            if (threadIdx.x < 32) {
-                const int lane = threadIdx.x;
-                unsigned loc[NS];
-                unsigned s = 0, npop = 0;
+        tiles_loop(k, [&](const CaseDev<S, A> &C, const MapScalars &SC, const MapScalarsF &SF, int a) {
+            stream_fast_group<BATCH_FAST_G>(C.M, C.MS, SC, SF, C.K, C.st, a);
+        });
+        if (!grid_barrier(g, cases, B)) return;
+        // the exact path over every case's work list (kb_slow's numbering)
+        if (threadIdx.x < 32) {
+            const int lane = threadIdx.x;
+            unsigned loc[NS];
+            unsigned s = 0, npop = 0;
+#pragma unroll
+            for (int i = 0; i < NS; ++i) {
+                loc[i] = lane < B ? *(volatile unsigned *)(cases[lane].st.wcount + i) : 0u;
+                s += loc[i];
+                if (i < NQ) npop += loc[i];
+            }
+            unsigned incl = s;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            if (lane < B) {
+                unsigned run = incl - s;
 #pragma unroll
                 for (int i = 0; i < NS; ++i) {
-                    loc[i] = lane < B ? *(volatile unsigned *)(cases[lane].st.wcount + i) : 0u;
-                    s += loc[i];
-                    if (i < NQ) npop += loc[i];
+                    pre[lane * NS + i] = run;
+                    run += loc[i];
                 }
-                unsigned incl = s;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += v;
-                }
-                if (lane < B) {
-                    unsigned run = incl - s;
-#pragma unroll
-                    for (int i = 0; i < NS; ++i) {
-                        pre[lane * NS + i] = run;
-                        run += loc[i];
-                    }
-                    if (lane == B - 1) pre[B * NS] = run;
-                    if (npop && blockIdx.x == 0 && cases[lane].stats)
-                        atomicAdd(cases[lane].stats, (unsigned long long)npop);
-                }
+                if (lane == B - 1) pre[B * NS] = run;
+                if (blockIdx.x == 0 && cases[lane].stats)
+                    atomicAdd(cases[lane].stats, step_count<S>(cases[lane].M, cases[lane].K.flags, npop));
             }
-            __syncthreads();
-            const unsigned total = pre[B * NS];
-            for (unsigned w = spread_first(); w < total; w += spread_stride()) {
-                int lo = 0, hi = B * NS - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (pre[mid] <= w) lo = mid;
-                    else hi = mid - 1;
-                }
-                const int c = lo / NS, i = lo % NS;
-                const CaseDev<S, A> &C = cases[c];
-                const int entry = C.st.work[(size_t)i * C.M.N + (w - pre[lo])];
-                if (i < NQ) {
-                    stream_slow_item(C.M, C.MS, sc[c], sf[c], sc[c], sf[c], C.K, C.st, C.err, entry);
-                } else {
-                    const unsigned mask = C.st.wmask[entry] & WMASK_DIRS;
-                    if (C.stats) atomicAdd(C.stats, (unsigned long long)__popc(mask));
-                    stream_bc_node<S, A>(C.M, C.MS, sc[c], sf[c], C.K, C.st, entry,
-                                         fast_map(C.MS, sf[c], entry, C.M.Xf[entry]), mask);
-                }
-            }
-            if (!grid_barrier(g, cases, B)) return;
-            tiles_loop(k, [&](const CaseDev<S, A> &C, const MapScalars &, const MapScalarsF &, int a) {
-                if (a <= NQ) C.st.wcount[a] = 0u; // the case's work list has been consumed
-                if (a < C.M.N) moments_node(C.K, C.st, C.M.N, C.err, a);
-            });
-        } else {
-            tiles_loop(k, [&](const CaseDev<S, A> &C, const MapScalars &SC, const MapScalarsF &, int a) {
-                if (a < C.M.N) stream_plain_node(C.M, C.MS, SC, SC, C.K, C.st, C.err, C.stats, a);
-            });
         }
+        __syncthreads();
+        const unsigned total = pre[B * NS];
+        for (unsigned w = spread_first(); w < total; w += spread_stride()) {
+            int lo = 0, hi = B * NS - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (pre[mid] <= w) lo = mid;
+                else hi = mid - 1;
+            }
+            const int c = lo / NS, i = lo % NS;
+            const CaseDev<S, A> &C = cases[c];
+            const int entry = C.st.work[(size_t)i * C.M.N + (w - pre[lo])];
+            if (i < NQ) {
+                const bool own = stream_slow_item(C.M, C.MS, sc[c], sf[c], sc[c], sf[c], C.K, C.st, C.err, entry);
+                count_own<S>(C.stats, own);
+            } else {
+                const unsigned mask = C.st.wmask[entry] & WMASK_DIRS;
+                count_wall<S>(C.stats, mask);
+                stream_bc_node<S, A>(C.M, C.MS, sc[c], sf[c], C.K, C.st, entry,
+                                     fast_map(C.MS, sf[c], entry, C.M.Xf[entry]), mask);
+            }
+        }
+        if (!grid_barrier(g, cases, B)) return;
+        tiles_loop(k, [&](const CaseDev<S, A> &C, const MapScalars &, const MapScalarsF &, int a) {
+            if (a <= NQ) C.st.wcount[a] = 0u; // the case's work list has been consumed
+            if (a < C.M.N) moments_node(C.K, C.st, C.M.N, C.err, a);
+        });
         if (!grid_barrier(g, cases, B)) return;
         tiles_loop(k, [&](const CaseDev<S, A> &C, const MapScalars &SC, const MapScalarsF &SF, int a) {
             if (a < C.M.N) deriv1_node<S, A, FAST>(C.M, C.MS, SC, SF, C.st, a);
@@ -796,16 +778,12 @@ void drop_graphs(alelb_batch *b)
 }
 
 // Phase kernels of one step, in order.
-int step_sequence(const alelb_batch *b, int seq[KT_N])
+int step_sequence(int seq[KT_N])
 {
     int n = 0;
-    if (b->prec == ALELB_PREC_FP32_DEV) {
-        seq[n++] = KT_FAST;
-        seq[n++] = KT_SLOW;
-        seq[n++] = KT_MOMENTS;
-    } else {
-        seq[n++] = KT_STREAM;
-    }
+    seq[n++] = KT_FAST;
+    seq[n++] = KT_SLOW;
+    seq[n++] = KT_MOMENTS;
     seq[n++] = KT_DERIV1;
     seq[n++] = KT_COLLIDE;
     return n;
@@ -866,9 +844,6 @@ void launch_phase(alelb_batch *b, const Part &P, int kt, int bs, int grid, int k
     const int B = P.B;
     const bool fast = b->prec == ALELB_PREC_FP32_DEV;
     switch (kt) {
-    case KT_STREAM:
-        launch_after(P.pdl, kb_stream<S, A>, dim3(tiles), dim3(bs), P.stream, cases, off, B, sc, count);
-        break;
     case KT_FAST:
         // fast_g: directions per thread, plus FAST_FUSED for the propagation
         // fused with the moments
@@ -890,11 +865,11 @@ void launch_phase(alelb_batch *b, const Part &P, int kt, int bs, int grid, int k
                     launch_after(P.pdl, kb_fast_fused<9, 256>, dim3(tiles), dim3(256), P.stream, cf, off, B, sf);
             }
         } else if (fast_g == 1)
-            launch_after(P.pdl, kb_fast<S, A, 1>, dim3(tiles, NQ), dim3(bs), P.stream, cases, off, B, sf);
+            launch_after(P.pdl, kb_fast<S, A, 1>, dim3(tiles, NQ), dim3(bs), P.stream, cases, off, B, sc, sf);
         else if (fast_g == 3)
-            launch_after(P.pdl, kb_fast<S, A, 3>, dim3(tiles, NQ / 3), dim3(bs), P.stream, cases, off, B, sf);
+            launch_after(P.pdl, kb_fast<S, A, 3>, dim3(tiles, NQ / 3), dim3(bs), P.stream, cases, off, B, sc, sf);
         else
-            launch_after(P.pdl, kb_fast<S, A, 9>, dim3(tiles, 1), dim3(bs), P.stream, cases, off, B, sf);
+            launch_after(P.pdl, kb_fast<S, A, 9>, dim3(tiles, 1), dim3(bs), P.stream, cases, off, B, sc, sf);
         break;
     case KT_SLOW:
         launch_after(P.pdl, kb_slow<S, A>, dim3(grid), dim3(bs), P.stream, cases, B, sc, sf, count);
@@ -974,7 +949,7 @@ template <class S, class A> int persistent_grid_t(int bs, int n_sm)
 void enqueue_step(alelb_batch *b, int k)
 {
     int seq[KT_N];
-    const int ns = step_sequence(b, seq);
+    const int ns = step_sequence(seq);
     for (int q = 0; q < ns; ++q) {
         const int kt = seq[q];
         cudaEvent_t ea = nullptr, eb = nullptr;
@@ -1000,7 +975,7 @@ void enqueue_step(alelb_batch *b, int k)
 cudaError_t enqueue_groups(alelb_batch *b, int k)
 {
     int seq[KT_N];
-    const int ns = step_sequence(b, seq);
+    const int ns = step_sequence(seq);
     const int lead = std::min(b->pipe ? (b->pipe == 2 ? 2 : 1) : 0, ns);
     cudaError_t st = cudaSuccess;
     for (int g = 0; g < b->groups && st == cudaSuccess; ++g) {
@@ -1493,7 +1468,7 @@ extern "C" alelb_status alelb_batch_tune(alelb_batch *b, int32_t reps, int32_t c
     if (st == cudaSuccess) st = cudaEventCreate(&e1);
     if (st != cudaSuccess) return bfail(b, st, "batch_tune");
     int seq[KT_N];
-    const int ns = step_sequence(b, seq);
+    const int ns = step_sequence(seq);
     const auto clear = [b]() {
         if (b->prec == ALELB_PREC_FP32_DEV)
             kb_clear_work<float, float>
@@ -1726,7 +1701,7 @@ extern "C" alelb_status alelb_batch_step_host(alelb_batch *b, const float *const
     cudaError_t st = stage_scalars(b, 0, 1); // the map scalars of time t_c + 1
     if (st == cudaSuccess) st = cudaEventRecord(b->gev_fork, b->stream);
     int seq[KT_N];
-    const int ns = step_sequence(b, seq);
+    const int ns = step_sequence(seq);
     for (int g = 0; g < P && st == cudaSuccess; ++g) {
         Part G = part(g);
         // the group's uploads, after the previous group's

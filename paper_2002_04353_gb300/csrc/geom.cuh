@@ -513,6 +513,7 @@ struct MeshDev {
     const float2 *nscale;  // (length scale, number of own elements) per node
     const uint8_t *bkind;  // [N] boundary kind of the node (0 interior)
     const uint8_t *vzero;  // [N] 1: mesh velocity exactly zero at all times
+    int nvzero;            // number of those nodes
     const float4 *cone;    // [N] boundary node: outgoing, incoming boundary edge (domain on the left)
     const uint8_t *conek;  // [N] kind of those edges (0 when the node has no such pair), | 4 at a
                            // convex corner of the domain, | 8 at a reflex one
@@ -522,6 +523,7 @@ struct MeshDev {
     const double2 *wall_nrm; // [NW] unit wall normal into the fluid, computational frame
     const int *orig_elem;  // [E] original element id
     const float4 *ejf;     // [2E] FP32 edge vectors (v1-v0, v2-v0) and inverse Jacobian rows
+    const double2 *ejd;    // [2E] inverse Jacobian rows in FP64 (grad xi, grad eta)
     const float *bdist;    // [N] lower bound of the node's distance to the nearest boundary edge
     const float4 *Xf;      // [N] node coordinates split hi + lo in FP32 (xh, yh, xl, yl)
     const float4 *v0f;     // [E] first frame vertex split hi + lo in FP32

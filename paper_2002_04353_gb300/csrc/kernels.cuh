@@ -1,23 +1,30 @@
 // kernels.cuh -- the kernels of one time step plus the element-choice
-// report and the force reduction.  The plain FP64 form:
+// report and the force reduction:
 //
-//   k_stream   propagation (Eq. Propagation): transformed velocities,
-//              departure points, element walk, P2 interpolation of the
-//              post-collision populations, Grad-type missing populations
-//              (Sec. IV.A); then moments, Q'_aaa (Eq. DeviationTerms) and
-//              mu/(rho T)
+//   k_stream_fast, k_stream_slow, k_moments   propagation (Eq. Propagation)
+//              in two passes, then the moments (described below; the
+//              FP64 form runs them with FP64 departure points and values)
 //   k_deriv1   D_a = (mu/rho T) d_a Q'_aaa in the owner element (Eq. Xa,
 //              Eqs. Ph_Derivative / FE_Derivative)
 //   k_collide  X_a = -d_a D_a, then the collision of Eqs. feqn/geqn
 //
-// and the deviation forms' propagation (k_stream_fast, k_stream_slow,
-// k_moments, below), which share k_deriv1 and k_collide.  One thread per
-// node unless noted.  Populations are stored by direction: FP64 buffers
+// and the plain FP64 propagation:
+//
+//   k_stream   transformed velocities, departure points, element walk, P2
+//              interpolation of the post-collision populations, Grad-type
+//              missing populations (Sec. IV.A); then moments, Q'_aaa (Eq.
+//              DeviationTerms) and mu/(rho T).  It serves the step that
+//              keeps no state of its own (no element cache) and the departure
+//              points that no FP32 certificate covers.
+//
+// One thread per node unless noted.  Populations are stored by direction: FP64 buffers
 // as pop[q * N + node] with q = 0..8 for f and 9..17 for g, the deviation
 // forms as (f_i, g_i) pairs, pop[2 (i N + node) + {0, 1}] (fg_get).
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "geom.cuh"
 #include "kinetic.cuh"
@@ -244,6 +251,152 @@ __device__ __forceinline__ void owner_grad_linear(const MeshDev &M, int a, const
     KY = (-x_eta * sxi + x_xi * seta) / detJ;
 }
 
+// Missing populations of Sec. IV.A at node a as the FP64 form computes them
+// (all nine directions), from its metrics and mesh velocity at the arrival
+// time: FP64 metrics and first-order FP64 gradients.
+template <class S, class A>
+__device__ __forceinline__ void missing_plain(const MeshDev &M, const KinParams<A> &K, const StateDev<S> &st, int a,
+                                              double a11, double a12, double a21, double a22, double Vx, double Vy,
+                                              A fm[NQ], A gm[NQ])
+{
+    // targets (Sec. IV.A): wall node -> u = V_G, rho and T at the
+    // probe point B; other nodes -> their previous-step fields
+    A rt, uxt, uyt, Tt;
+    const int wi = M.wall_idx[a];
+    if (wi >= 0) {
+        const int pe = M.probe_e[wi];
+        const double2 pxi = M.probe_xi[wi];
+        A Nw[6];
+        shape6<A>((A)pxi.x, (A)pxi.y, Nw);
+        A r = 0, t = 0, ub = 0, vb = 0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            int b = M.conn[6 * pe + k];
+            r += Nw[k] * (A)st.rho[b];
+            t += Nw[k] * (A)st.T[b];
+            if (K.flags & FLAG_SLIP) {
+                ub += Nw[k] * (A)st.ux[b];
+                vb += Nw[k] * (A)st.uy[b];
+            }
+        }
+        rt = r;
+        Tt = t;
+        uxt = (A)Vx;
+        uyt = (A)Vy;
+        if (K.flags & FLAG_SLIP) {
+            const double2 nw = M.wall_nrm[wi];
+            slip_target<A>((A)a11, (A)a12, (A)a21, (A)a22, (A)nw.x, (A)nw.y, ub, vb, (A)Vx, (A)Vy, uxt, uyt);
+        }
+    } else {
+        // off-wall node: its previous-step fields; the velocity is the
+        // mesh velocity instead under FLAG_OFFWALL_VG
+        const bool vg = (K.flags & FLAG_OFFWALL_VG) != 0;
+        rt = (A)st.rho[a];
+        uxt = vg ? (A)Vx : (A)st.ux[a];
+        uyt = vg ? (A)Vy : (A)st.uy[a];
+        Tt = (A)st.T[a];
+    }
+    A du[4] = {0, 0, 0, 0}, dT[2] = {0, 0};
+    if (!(K.flags & FLAG_BC_EQ) && !((K.flags & FLAG_SLIP) && wi >= 0)) {
+        double KX, KY;
+        owner_grad_linear(M, a, st.ux, KX, KY);
+        du[0] = (A)(a11 * KX + a21 * KY);
+        du[1] = (A)(a12 * KX + a22 * KY);
+        owner_grad_linear(M, a, st.uy, KX, KY);
+        du[2] = (A)(a11 * KX + a21 * KY);
+        du[3] = (A)(a12 * KX + a22 * KY);
+        owner_grad_linear(M, a, st.T, KX, KY);
+        dT[0] = (A)(a11 * KX + a21 * KY);
+        dT[1] = (A)(a12 * KX + a22 * KY);
+    }
+    grad_missing(K, rt, uxt, uyt, Tt, du, dT, fm, gm);
+}
+
+// ---------------------------------------------------------------------------
+// Departure point and interpolation of the FP64 form, shared by its fast and
+// its exact path.  Every operation that rounds is written as an intrinsic,
+// which the compiler neither fuses nor reorders: a population's value is the
+// same bits whichever kernel settles it, so it depends neither on the element
+// cache nor on the batching.
+// ---------------------------------------------------------------------------
+struct Node64 {
+    double a11, a12, a21, a22, wx, wy; // A = g^{-1,T}, w = A (V_G - U) of a node
+};
+
+// TR: the map is a translation (no map, plunge): A = I and w is the same at
+// every node, so no FP64 operation runs per node but the two subtractions.
+template <bool TR>
+__device__ __forceinline__ Node64 node64(const MapStatic &MS, const MapScalars &sc, int a, double2 X, bool literal)
+{
+    Node64 n;
+    if (TR) {
+        n.a11 = n.a22 = 1.0;
+        n.a12 = n.a21 = 0.0;
+        n.wx = ds(0.0, sc.Ux);
+        n.wy = ds(sc.vy, sc.Uy); // vy is zero without a map
+        return n;
+    }
+    double xX, xY, yX, yY, Vx, Vy;
+    map_node(MS, sc, a, X.x, X.y, xX, xY, yX, yY, Vx, Vy);
+    metric_inverse_T(xX, xY, yX, yY, n.a11, n.a12, n.a21, n.a22);
+    mesh_velocity_term(n.a11, n.a12, n.a21, n.a22, ds(Vx, sc.Ux), ds(Vy, sc.Uy), literal, n.wx, n.wy);
+    return n;
+}
+
+// a cx + b cy for cx, cy in {-1, 0, 1}: the value of da(dm(a, cx), dm(b, cy))
+// (the products are exact, a zero term adds nothing) in at most one FP64
+// operation.
+__device__ __forceinline__ double lattice_sum(double a, double b, int cx, int cy)
+{
+    const double u = cx < 0 ? -a : a, v = cy < 0 ? -b : b;
+    return cx == 0 ? (cy == 0 ? 0.0 : v) : (cy == 0 ? u : da(u, v));
+}
+
+// The canonical departure point (departure() in geom.cuh) of population i.
+template <bool TR>
+__device__ __forceinline__ void departure64(const Node64 &n, int i, double2 X, double &px, double &py)
+{
+    const int cx = lat_cx(i), cy = lat_cy(i);
+    px = ds(X.x, ds(TR ? (double)cx : lattice_sum(n.a11, n.a12, cx, cy), n.wx));
+    py = ds(X.y, ds(TR ? (double)cy : lattice_sum(n.a21, n.a22, cx, cy), n.wy));
+}
+
+// The pair (f_i, g_i) interpolated at p in element e (frame shift sx, sy):
+// local coordinates through the element's stored FP64 inverse Jacobian, the
+// six shape functions, six gathers.
+__device__ __forceinline__ void interp64(const MeshDev &M, const double *post, int N, int i, int e, int sx, int sy,
+                                         double px, double py, double &f, double &g)
+{
+    int nb[6]; // the six node numbers in three 8-byte loads
+    const int2 *cp = reinterpret_cast<const int2 *>(M.conn + 6 * e);
+#pragma unroll
+    for (int h = 0; h < 3; ++h) {
+        const int2 v = cp[h];
+        nb[2 * h] = v.x;
+        nb[2 * h + 1] = v.y;
+    }
+    double2 v0 = M.ev[3 * e];
+    const double2 j1 = M.ejd[2 * e], j2 = M.ejd[2 * e + 1];
+    if (sx) v0.x = da(v0.x, sx * M.Lx);
+    if (sy) v0.y = da(v0.y, sy * M.Ly);
+    const double dx = ds(px, v0.x), dy = ds(py, v0.y);
+    const double xi = dfma(j1.x, dx, dm(j1.y, dy)), eta = dfma(j2.x, dx, dm(j2.y, dy));
+    const double l0 = ds(ds(1.0, xi), eta);
+    const double q = dm(4.0, xi), r = dm(4.0, eta);
+    const double w[6] = {dm(l0, dfma(2.0, l0, -1.0)), dm(xi, dfma(2.0, xi, -1.0)), dm(eta, dfma(2.0, eta, -1.0)),
+                         dm(q, l0), dm(q, eta), dm(r, l0)};
+    double fb, gb;
+    fg_get(post, i, nb[0], N, fb, gb);
+    f = dm(w[0], fb);
+    g = dm(w[0], gb);
+#pragma unroll
+    for (int k = 1; k < 6; ++k) {
+        fg_get(post, i, nb[k], N, fb, gb);
+        f = dfma(w[k], fb, f);
+        g = dfma(w[k], gb, g);
+    }
+}
+
 // The plain FP64 propagation: every population through the FP64 departure
 // point and the exact walk, one thread per node.
 // scd: map scalars of the transformed velocities (sc, or those of the
@@ -328,59 +481,7 @@ __device__ __forceinline__ void stream_plain_node(const MeshDev &M, const MapSta
             metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
         }
         A fm[NQ], gm[NQ];
-        if (miss & ~far) {
-            // targets (Sec. IV.A): wall node -> u = V_G, rho and T at the
-            // probe point B; other nodes -> their previous-step fields
-            A rt, uxt, uyt, Tt;
-            const int wi = M.wall_idx[a];
-            if (wi >= 0) {
-                const int pe = M.probe_e[wi];
-                const double2 pxi = M.probe_xi[wi];
-                A Nw[6];
-                shape6<A>((A)pxi.x, (A)pxi.y, Nw);
-                A r = 0, t = 0, ub = 0, vb = 0;
-#pragma unroll
-                for (int k = 0; k < 6; ++k) {
-                    int b = M.conn[6 * pe + k];
-                    r += Nw[k] * (A)st.rho[b];
-                    t += Nw[k] * (A)st.T[b];
-                    if (K.flags & FLAG_SLIP) {
-                        ub += Nw[k] * (A)st.ux[b];
-                        vb += Nw[k] * (A)st.uy[b];
-                    }
-                }
-                rt = r;
-                Tt = t;
-                uxt = (A)Vx;
-                uyt = (A)Vy;
-                if (K.flags & FLAG_SLIP) {
-                    const double2 nw = M.wall_nrm[wi];
-                    slip_target<A>((A)a11, (A)a12, (A)a21, (A)a22, (A)nw.x, (A)nw.y, ub, vb, (A)Vx, (A)Vy, uxt, uyt);
-                }
-            } else {
-                // off-wall node: its previous-step fields; the velocity is the
-                // mesh velocity instead under FLAG_OFFWALL_VG
-                const bool vg = (K.flags & FLAG_OFFWALL_VG) != 0;
-                rt = (A)st.rho[a];
-                uxt = vg ? (A)Vx : (A)st.ux[a];
-                uyt = vg ? (A)Vy : (A)st.uy[a];
-                Tt = (A)st.T[a];
-            }
-            A du[4] = {0, 0, 0, 0}, dT[2] = {0, 0};
-            if (!(K.flags & FLAG_BC_EQ) && !((K.flags & FLAG_SLIP) && wi >= 0)) {
-                double KX, KY;
-                owner_grad_linear(M, a, st.ux, KX, KY);
-                du[0] = (A)(a11 * KX + a21 * KY);
-                du[1] = (A)(a12 * KX + a22 * KY);
-                owner_grad_linear(M, a, st.uy, KX, KY);
-                du[2] = (A)(a11 * KX + a21 * KY);
-                du[3] = (A)(a12 * KX + a22 * KY);
-                owner_grad_linear(M, a, st.T, KX, KY);
-                dT[0] = (A)(a11 * KX + a21 * KY);
-                dT[1] = (A)(a12 * KX + a22 * KY);
-            }
-            grad_missing(K, rt, uxt, uyt, Tt, du, dT, fm, gm);
-        }
+        if (miss & ~far) missing_plain(M, K, st, a, a11, a12, a21, a22, Vx, Vy, fm, gm);
 #pragma unroll
         for (int i = 0; i < NQ; ++i) {
             if (!(miss >> i & 1)) continue;
@@ -418,8 +519,10 @@ __global__ void __launch_bounds__(128) k_stream(MeshDev M, MapStatic MS, MapScal
 }
 
 // ---------------------------------------------------------------------------
-// The deviation-form propagation, split by path so that the rare exact
-// work does not stall the warps of the common case:
+// The propagation, split by path so that the rare exact work does not
+// stall the warps of the common case (FP64 form, 150,400-node plunge: 103 +
+// 43 + 31 us for the three kernels against 1,194 us in one pass with every
+// population walked in FP64; 9,216-node box 20 + 28 + 12 against 268 us):
 //   k_stream_fast  per population: FP32 map; a population whose
 //                  previous-step element is verified (fast_decide) is
 //                  interpolated and stored, one certified missing by the
@@ -447,6 +550,18 @@ __device__ __forceinline__ void stream_bc_node(const MeshDev &M, const MapStatic
                                                const FastMap &F, unsigned mask)
 {
     const int N = M.N;
+    if constexpr (std::is_same<S, double>::value) { // FP64 metrics and gradients
+        const double2 X = M.X[a];
+        double xX, xY, yX, yY, vx, vy, b11, b12, b21, b22;
+        map_node(MS, sc, a, X.x, X.y, xX, xY, yX, yY, vx, vy);
+        metric_inverse_T(xX, xY, yX, yY, b11, b12, b21, b22);
+        A fm[NQ], gm[NQ];
+        missing_plain(M, K, st, a, b11, b12, b21, b22, vx, vy, fm, gm);
+#pragma unroll
+        for (int i = 0; i < NQ; ++i)
+            if (mask >> i & 1u) fg_put(st.str, i, a, N, fm[i], gm[i]);
+        return;
+    }
     float a11, a12, a21, a22, Vx, Vy;
     if (F.ok) {
         a11 = F.A11;
@@ -628,12 +743,65 @@ __device__ __forceinline__ void append_pop(const StateDev<S> &st, int a, int N, 
 #define ALELB_BATCH_FAST_G 9
 #endif
 constexpr int FAST_G = ALELB_FAST_G, BATCH_FAST_G = ALELB_BATCH_FAST_G, FAST_G_NODES = 300000;
+// The FP64 form's, by nodes, when the map is not a translation (the rule
+// with its timings stands at the launch).
+constexpr int FAST64_G3_NODES = 8192, FAST64_G9_NODES = 65536;
 static_assert(NQ % FAST_G == 0 && NQ % BATCH_FAST_G == 0, "directions per thread");
 
+// The FP64 form's populations i0 .. i0 + G - 1 of node a: the decision is the
+// deviation forms' certified FP32 one (the previous-step element, else the
+// exterior cone), the departure point and the interpolation of an accepted
+// population run in FP64 (codes as stream_fast_pop's).  Bound by the FP64
+// pipe (two lanes per SM and clock): 36 FP64 operations per population, so
+// the element search and its predicates stay off that pipe.
+template <int G, bool TR>
+__device__ __forceinline__ void stream_fast_pops64(const MeshDev &M, const MapStatic &MS, const MapScalars &sc,
+                                                   const MapScalarsF &sf, const KinParams<double> &K,
+                                                   const StateDev<double> &st, int a, int i0, int code[G])
+{
+    const int N = M.N;
+    int c[G];
+#pragma unroll
+    for (int j = 0; j < G; ++j) c[j] = st.cache[(i0 + j) * N + a];
+    const float bd = M.bdist[a];
+    const float4 Xf = M.Xf[a];
+    const double2 X = M.X[a];
+    FastMap F = TR ? fast_map_translation(sf, Xf) : fast_map(MS, sf, a, Xf);
+    if (K.flags & (FLAG_LITERAL_VG | FLAG_EXACT_CHAR)) F.ok = false;
+    const Node64 n = node64<TR>(MS, sc, a, X, false);
+#pragma unroll
+    for (int j = 0; j < G; ++j) {
+        const int i = i0 + j;
+        if (i == 0 && M.vzero[a] && !(K.flags & FLAG_SHIFT)) { // c^_0 exactly zero: the node's own value
+            fg_copy(st.str, st.post, 0, a, N);
+            code[j] = 0;
+            continue;
+        }
+        if (!F.ok) {
+            code[j] = 1;
+            continue;
+        }
+        int e;
+        float xi, eta;
+        if (fast_decide(M, F, Xf, bd, a, i, c[j], e, xi, eta)) {
+            double px, py, f, g;
+            departure64<TR>(n, i, X, px, py);
+            interp64(M, st.post, N, i, e, 0, 0, px, py, f, g);
+            fg_put(st.str, i, a, N, f, g);
+            code[j] = 0;
+            continue;
+        }
+        const int ck = cone_missing(M, F, a, i);
+        if (ck == 2) fg_put(st.str, i, a, N, K.finf[i], K.ginf[i]); // far field: free-stream equilibria
+        code[j] = ck == 2 ? 0 : ck == 1 ? 2 : 1;
+    }
+}
+
 // Populations G y .. G y + G - 1 of node a (y = blockIdx.y): settled, or
-// entered in the work list.
+// entered in the work list.  sc, sf: the map of the transformed velocities
+// (sc is read by the FP64 form only).
 template <int G, class S, class A, bool TR = false>
-__device__ __forceinline__ void stream_fast_group(const MeshDev &M, const MapStatic &MS,
+__device__ __forceinline__ void stream_fast_group(const MeshDev &M, const MapStatic &MS, const MapScalars &sc,
                                                   const MapScalarsF &sf, const KinParams<A> &K,
                                                   const StateDev<S> &st, int a)
 {
@@ -641,7 +809,9 @@ __device__ __forceinline__ void stream_fast_group(const MeshDev &M, const MapSta
     int code[G];
 #pragma unroll
     for (int j = 0; j < G; ++j) code[j] = 0;
-    if (a < M.N) {
+    if constexpr (std::is_same<S, double>::value) {
+        if (a < M.N) stream_fast_pops64<G, TR>(M, MS, sc, sf, K, st, a, i0, code);
+    } else if (a < M.N) {
         // the loads of the thread's cache entries go out together (the
         // stores of the populations would otherwise order them one by one)
         int c[G];
@@ -674,11 +844,11 @@ constexpr int FAST_BS = ALELB_FAST_BS;
 // Grid (node blocks, 9 / G direction groups).  TR: the map is a
 // translation (no map, plunge).
 template <class S, class A, int G, bool TR>
-__global__ void __launch_bounds__(FAST_BS) k_stream_fast(MeshDev M, MapStatic MS, MapScalarsF sf,
+__global__ void __launch_bounds__(FAST_BS) k_stream_fast(MeshDev M, MapStatic MS, MapScalars sc, MapScalarsF sf,
                                                      KinParams<A> K, StateDev<S> st)
 {
     wait_prior_grid();
-    stream_fast_group<G, S, A, TR>(M, MS, sf, K, st, blockIdx.x * blockDim.x + threadIdx.x);
+    stream_fast_group<G, S, A, TR>(M, MS, sc, sf, K, st, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // One listed population (code = 9 node + direction): exact decision, then
@@ -690,8 +860,9 @@ __global__ void __launch_bounds__(FAST_BS) k_stream_fast(MeshDev M, MapStatic MS
 // sc, sf: the map at the arrival time (wall condition); scd, sfd: the map
 // of the transformed velocities (the same, or the midpoint time under
 // FLAG_MIDPOINT).
+// Returns true when c^ is exactly zero (the population is the node's own).
 template <class S, class A>
-__device__ __forceinline__ void stream_slow_item(const MeshDev &M, const MapStatic &MS,
+__device__ __forceinline__ bool stream_slow_item(const MeshDev &M, const MapStatic &MS,
                                                  const MapScalars &sc, const MapScalarsF &sf,
                                                  const MapScalars &scd, const MapScalarsF &sfd,
                                                  const KinParams<A> &K, const StateDev<S> &st,
@@ -728,11 +899,11 @@ __device__ __forceinline__ void stream_slow_item(const MeshDev &M, const MapStat
         const int ck = F.ok && !literal ? certified_missing(M, F, a, i, &clear) : 0;
         if (ck == 1) { // certified to meet a wall first
             stream_bc_node<S, A>(M, MS, sc, sf, K, st, a, Fb, 1u << i);
-            return;
+            return false;
         }
         if (ck == 2) { // certified to leave through the far field
             fg_put(st.str, i, a, N, K.finf[i], K.ginf[i]);
-            return;
+            return false;
         }
         Loc L;
         int pe;
@@ -769,25 +940,34 @@ __device__ __forceinline__ void stream_slow_item(const MeshDev &M, const MapStat
         } else if (L.e >= 0) {
             const int e = L.e;
             st.cache[i * N + a] = cache_code(M, e, L.sx, L.sy, a);
-            const float4 J = M.ejf[2 * e + 1];
-            A Nw[6];
-            shape6<A>((A)(J.x * qx + J.y * qy), (A)(J.z * qx + J.w * qy), Nw);
+            if constexpr (std::is_same<S, double>::value) {
+                const double2 X = M.X[a];
+                const Node64 n = node64<false>(MS, scd, a, X, literal != 0);
+                double px, py;
+                departure64<false>(n, i, X, px, py);
+                interp64(M, st.post, N, i, e, L.sx, L.sy, px, py, fi, gi);
+            } else {
+                const float4 J = M.ejf[2 * e + 1];
+                A Nw[6];
+                shape6<A>((A)(J.x * qx + J.y * qy), (A)(J.z * qx + J.w * qy), Nw);
 #pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                const int b = M.conn[6 * e + k];
-                A fb, gb;
-                fg_get(st.post, i, b, N, fb, gb);
-                fi += Nw[k] * fb;
-                gi += Nw[k] * gb;
+                for (int k = 0; k < 6; ++k) {
+                    const int b = M.conn[6 * e + k];
+                    A fb, gb;
+                    fg_get(st.post, i, b, N, fb, gb);
+                    fi += Nw[k] * fb;
+                    gi += Nw[k] * gb;
+                }
             }
         } else if (L.kind == 2) {
             fi = K.finf[i];
             gi = K.ginf[i];
         } else {
             stream_bc_node<S, A>(M, MS, sc, sf, K, st, a, Fb, 1u << i);
-            return;
+            return false;
         }
         fg_put(st.str, i, a, N, fi, gi);
+        return L.e == -2;
     }
 }
 
@@ -802,6 +982,26 @@ __device__ __forceinline__ unsigned spread_first()
 }
 __device__ __forceinline__ unsigned spread_stride() { return gridDim.x * blockDim.x; }
 
+// The counter of alelb_info.  The deviation forms count the populations left
+// to the exact path (the listed ones and the wall nodes' masked directions);
+// the FP64 form counts every population that is located, which is all 9 N
+// less those whose c^ is exactly zero: the nodes of zero mesh velocity (known
+// per mesh) and the ones that the exact path meets.
+template <class S>
+__device__ __forceinline__ unsigned long long step_count(const MeshDev &M, int flags, unsigned listed)
+{
+    if (!std::is_same<S, double>::value) return listed;
+    return (unsigned long long)NQ * M.N - (flags & FLAG_SHIFT ? 0 : M.nvzero);
+}
+template <class S> __device__ __forceinline__ void count_wall(unsigned long long *stats, unsigned mask)
+{
+    if (!std::is_same<S, double>::value && stats) atomicAdd(stats, (unsigned long long)__popc(mask));
+}
+template <class S> __device__ __forceinline__ void count_own(unsigned long long *stats, bool own)
+{
+    if (std::is_same<S, double>::value && stats && own) atomicAdd(stats, ~0ull); // one less
+}
+
 // Entry w of the exact path's numbering (work_prefix over the 10 segments):
 // a population (9 node + direction), or a listed wall node, whose wall
 // condition is computed once for all its certified directions.
@@ -814,12 +1014,13 @@ __device__ __forceinline__ void slow_entry(const MeshDev &M, const MapStatic &MS
                                            unsigned long long *stats)
 {
     if (w < pre[NQ]) {
-        stream_slow_item(M, MS, sc, sf, scd, sfd, K, st, err, work_at(st.work, M.N, pre, w),
-                         prop ? prop[w] : -1, prop && stats ? stats + 1 : nullptr);
+        const bool own = stream_slow_item(M, MS, sc, sf, scd, sfd, K, st, err, work_at(st.work, M.N, pre, w),
+                                          prop ? prop[w] : -1, prop && stats ? stats + 1 : nullptr);
+        count_own<S>(stats, own);
     } else {
         const int a = st.work[(size_t)NQ * M.N + (w - pre[NQ])];
         const unsigned mask = st.wmask[a] & WMASK_DIRS;
-        if (stats) atomicAdd(stats, (unsigned long long)__popc(mask));
+        count_wall<S>(stats, mask);
         stream_bc_node<S, A>(M, MS, sc, sf, K, st, a, fast_map(MS, sf, a, M.Xf[a]), mask);
     }
 }
@@ -836,7 +1037,7 @@ __global__ void __launch_bounds__(128) k_stream_slow(MeshDev M, MapStatic MS, Ma
     __syncthreads();
     const unsigned n = pre[NQ];
     const unsigned total = n + st.wcount[NQ];
-    if (stats && blockIdx.x == 0 && threadIdx.x == 0 && n) atomicAdd(stats, (unsigned long long)n);
+    if (stats && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(stats, step_count<S>(M, K.flags, n));
     for (unsigned w = spread_first(); w < total; w += spread_stride())
         slow_entry(M, MS, sc, sf, scd, sfd, K, st, err, pre, w, prop, stats);
 }

@@ -54,7 +54,7 @@ struct HostTables {
     int mkind = 0;
     double mp[16] = {0};
     std::vector<int> node_old2new, node_new2old, elem_old2new, elem_new2old;
-    std::vector<double2> X, ev, probe_xi, wall_nrm;
+    std::vector<double2> X, ev, probe_xi, wall_nrm, ejd;
     std::vector<int> nbr, conn, rank, orig, fan_ptr, wall_idx, probe_e, bcel, ring_ptr, ring;
     std::vector<float2> nscale;
     std::vector<uint32_t> einfo;
@@ -91,6 +91,7 @@ struct HostTables {
         D.bcel = bcel.data();
         D.bkind = bkind.data();
         D.vzero = vzero.data();
+        D.nvzero = (int)std::count(vzero.begin(), vzero.end(), (uint8_t)1);
         D.cone = cone.data();
         D.conek = conek.data();
         D.wall_idx = wall_idx.data();
@@ -99,6 +100,7 @@ struct HostTables {
         D.wall_nrm = wall_nrm.data();
         D.orig_elem = orig.data();
         D.ejf = ejf.data();
+        D.ejd = ejd.data();
         D.bdist = bdist.data();
         D.Xf = Xf.data();
         D.v0f = v0f.data();
@@ -609,10 +611,13 @@ inline alelb_status build_tables(const alelb_mesh_desc *d, HostTables &T, std::s
     // FP32 edge vectors and inverse Jacobians (interpolation weights and the
     // certified FP32 containment filter)
     T.ejf.assign((size_t)2 * E, make_float4(0, 0, 0, 0));
+    T.ejd.resize((size_t)2 * E);
     for (int en = 0; en < E; ++en) {
         double2 v0 = ev[3 * en], v1 = ev[3 * en + 1], v2 = ev[3 * en + 2];
         double e1x = v1.x - v0.x, e1y = v1.y - v0.y, e2x = v2.x - v0.x, e2y = v2.y - v0.y;
         double det = e1x * e2y - e2x * e1y;
+        T.ejd[2 * en] = make_double2(e2y / det, -e2x / det);
+        T.ejd[2 * en + 1] = make_double2(-e1y / det, e1x / det);
         T.ejf[2 * en] = make_float4((float)e1x, (float)e1y, (float)e2x, (float)e2y);
         T.ejf[2 * en + 1] = make_float4((float)(e2y / det), (float)(-e2x / det), (float)(-e1y / det),
                                         (float)(e1x / det));
