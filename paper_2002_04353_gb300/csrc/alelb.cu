@@ -470,11 +470,15 @@ cudaError_t launch_step(alelb_solver *s, StateDev<S> &st, KinParams<A> &K, const
                            : (s->flags & ALELB_FLAG_MIDPOINT) ? solver_map(s, map_scalars(m->T.mkind, m->T.mp, s->t + 0.5))
                                                               : sc;
     const MapScalarsF sfd = to_f32(scd, m->T);
+    // The two passes in every form; the FP64 form keeps the plain pass where
+    // no FP32 certificate covers the departure point, so that nothing would
+    // settle in the first one.
+    const bool passes = fast || !(s->flags & (ALELB_FLAG_LITERAL_VG | ALELB_FLAG_EXACT_CHAR));
     if (m->etype == ALELB_ELEM_Q2QUAD) { // quad.cu: propagation, moments, the two derivative passes
-        const int qseq64[4] = {KT_STREAM, KT_MOMENTS, KT_DERIV1, KT_COLLIDE};
-        const int qseq32[5] = {KT_FAST, KT_SLOW, KT_MOMENTS, KT_DERIV1, KT_COLLIDE};
-        const int *qseq = fast ? qseq32 : qseq64;
-        const int nq = fast ? 5 : 4;
+        const int seq1[4] = {KT_STREAM, KT_MOMENTS, KT_DERIV1, KT_COLLIDE};
+        const int seq2[5] = {KT_FAST, KT_SLOW, KT_MOMENTS, KT_DERIV1, KT_COLLIDE};
+        const int *qseq = passes ? seq2 : seq1;
+        const int nq = passes ? 5 : 4;
         for (int q = 0; q < nq; ++q) {
             if (qseq[q] == KT_DERIV1 && !phi) continue;
             cudaEvent_t ea = nullptr, eb = nullptr;
@@ -493,10 +497,6 @@ cudaError_t launch_step(alelb_solver *s, StateDev<S> &st, KinParams<A> &K, const
         return cudaGetLastError();
     }
     int seq[KT_N], ns = 0;
-    // The two passes in every form; the FP64 form keeps the plain pass where
-    // no FP32 certificate covers the departure point, so that nothing would
-    // settle in the first one.
-    const bool passes = fast || !(s->flags & (ALELB_FLAG_LITERAL_VG | ALELB_FLAG_EXACT_CHAR));
     if (passes) {
         seq[ns++] = KT_FAST;
         if (s->mlp) seq[ns++] = KT_PROPOSE;

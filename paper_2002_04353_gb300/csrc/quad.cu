@@ -4,12 +4,14 @@
 // missing populations) is the one the triangles use (kinetic.cuh); only the
 // geometry differs: the walk over quadrilaterals, Newton's method for the
 // local coordinates of Eq. NonLinear_Eq, the nine shape functions of
-// Eq. Propagation and the element gradients (quad.cuh).  The deviation
-// forms first try the previous-step element under a certified FP32 test
-// (quad_fast_decide); every other population, and every population of the
-// FP64 form, takes the exact FP64 path.
+// Eq. Propagation and the element gradients (quad.cuh).  Every form first
+// tries the previous-step element under a certified FP32 test
+// (quad_fast_decide); the other populations take the exact FP64 path.  The
+// FP64 form at 150,400 nodes (plunge): 225 + 67 us for the two passes against
+// 3,881 us with every population walked and Newton in FP64.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <string>
 #include <type_traits>
 
@@ -47,38 +49,44 @@ __device__ __forceinline__ bool quad_fast_pop(const QuadDev &M, const FastMap &F
     return true;
 }
 
-// Propagation of population pairs i0 .. i0 + G - 1 of node a (Eq.
-// Propagation over the nine nodes of the departure element) and, for those
-// that are missing, the condition of Sec. IV.A.  TRY: first the certified
-// FP32 decision (deviation forms).  The moments, Q'_aaa and mu/(rho T)
-// follow in k_moments, as on triangles.
-// Returns the number of element walks taken.
-template <int G, bool TRY, class S, class A>
-__device__ __forceinline__ unsigned quad_stream_pops(const QuadDev &M, const MapStatic &MS, const MapScalars &sc,
-                                                     const MapScalars &scd, const MapScalarsF &sfd,
-                                                     const KinParams<A> &K, const StateDev<S> &st, int *err, int a,
-                                                     int i0)
+// The FP64 form's population: the same certified decision, then departure
+// point, local coordinates and interpolation in FP64.
+template <bool TR>
+__device__ __forceinline__ bool quad_fast_pop64(const QuadDev &M, const FastMap &F, const Node64 &n, float4 Xf, double2 X,
+                                                const StateDev<double> &st, int a, int i, int c)
 {
-    constexpr bool FAST = !std::is_same<S, double>::value; // the deviation forms keep the element cache
+    int e;
+    float cw[8];
+    if (!quad_fast_decide(M, F, Xf, a, i, c, e, cw)) return false;
+    double px, py, xi, eta, f, g;
+    departure64<TR>(n, i, X, px, py);
+    if (!quad_local64(M, e, 0, 0, px, py, xi, eta)) return false;
+    quad_interp64(M, st.post, M.N, i, e, xi, eta, f, g);
+    fg_put(st.str, i, a, M.N, f, g);
+    return true;
+}
+
+// Propagation of population pairs i0 .. i0 + G - 1 of node a on the exact
+// path (Eq. Propagation over the nine nodes of the departure element) and,
+// for those that are missing, the condition of Sec. IV.A.  KEEP: the element
+// is kept for the next step's certified check.  The moments, Q'_aaa and
+// mu/(rho T) follow in k_moments, as on triangles.
+// Returns the number of element walks taken.
+template <int G, bool KEEP, class S, class A>
+__device__ __forceinline__ unsigned quad_stream_pops(const QuadDev &M, const MapStatic &MS, const MapScalars &sc,
+                                                     const MapScalars &scd, const KinParams<A> &K,
+                                                     const StateDev<S> &st, int *err, int a, int i0)
+{
     const int N = M.N;
     const double2 Xa = M.X[a];
     bool have64 = false;
     double a11 = 0, a12 = 0, a21 = 0, a22 = 0, wx = 0, wy = 0, Vx = 0, Vy = 0;
     int miss = 0, far = 0;
     unsigned walks = 0;
-    float4 Xf = make_float4(0.f, 0.f, 0.f, 0.f);
-    FastMap F;
-    F.ok = false;
-    if (FAST && TRY) {
-        Xf = M.Xf[a];
-        F = fast_map(MS, sfd, a, Xf);
-        if (K.flags & (FLAG_LITERAL_VG | FLAG_EXACT_CHAR)) F.ok = false;
-    }
 #pragma unroll 1
     for (int i = i0; i < i0 + G; ++i) {
         A fi = 0, gi = 0;
         int src = -1;
-        if (FAST && TRY && F.ok && quad_fast_pop<S, A>(M, F, Xf, st, a, i)) continue;
         if (!have64 && !(K.flags & FLAG_EXACT_CHAR)) {
             double xX, xY, yX, yY;
             map_node(MS, scd, a, Xa.x, Xa.y, xX, xY, yX, yY, Vx, Vy);
@@ -97,7 +105,7 @@ __device__ __forceinline__ unsigned quad_stream_pops(const QuadDev &M, const Map
         } else {
             ++walks;
             const Loc L = quad_walk(M, a, Xa.x, Xa.y, px, py, err);
-            if (FAST) // the element for the next step's certified check
+            if (KEEP) // the element for the next step's certified check
                 st.cache[i * N + a] = L.e >= 0 ? (L.e | ((L.sx + 1) << 28) | ((L.sy + 1) << 30)) : -1;
             if (L.e == -2) {
                 src = a;
@@ -108,17 +116,25 @@ __device__ __forceinline__ unsigned quad_stream_pops(const QuadDev &M, const Map
             } else if (L.vnode >= 0) {
                 src = L.vnode;
             } else {
-                A xi, eta;
-                if (!quad_local<A>(M, L.e, L.sx, L.sy, px, py, xi, eta)) set_err(err, ERR_LOCATE);
-                A Nw[9];
-                shape9<A>(xi, eta, Nw);
+                if constexpr (std::is_same<S, double>::value) {
+                    double xi, eta;
+                    if (!quad_local64(M, L.e, L.sx, L.sy, px, py, xi, eta) &&
+                        !quad_local<double>(M, L.e, L.sx, L.sy, px, py, xi, eta))
+                        set_err(err, ERR_LOCATE);
+                    quad_interp64(M, st.post, N, i, L.e, xi, eta, fi, gi);
+                } else {
+                    A xi, eta;
+                    if (!quad_local<A>(M, L.e, L.sx, L.sy, px, py, xi, eta)) set_err(err, ERR_LOCATE);
+                    A Nw[9];
+                    shape9<A>(xi, eta, Nw);
 #pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const int b = M.conn[9 * L.e + k];
-                    A fb, gb;
-                    fg_get(st.post, i, b, N, fb, gb);
-                    fi += Nw[k] * fb;
-                    gi += Nw[k] * gb;
+                    for (int k = 0; k < 9; ++k) {
+                        const int b = M.conn[9 * L.e + k];
+                        A fb, gb;
+                        fg_get(st.post, i, b, N, fb, gb);
+                        fi += Nw[k] * fb;
+                        gi += Nw[k] * gb;
+                    }
                 }
             }
         }
@@ -197,57 +213,94 @@ __device__ __forceinline__ unsigned quad_stream_pops(const QuadDev &M, const Map
 // Grid (node blocks, 9 / G direction groups): G directions per thread.
 template <class S, class A, int G>
 __global__ void __launch_bounds__(128) kq_stream(QuadDev M, MapStatic MS, MapScalars sc, MapScalars scd,
-                                                 MapScalarsF sfd, KinParams<A> K, StateDev<S> st, int *err,
+                                                 KinParams<A> K, StateDev<S> st, int *err,
                                                  unsigned long long *stats)
 {
     wait_prior_grid();
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned walks = 0;
-    if (a < M.N) walks = quad_stream_pops<G, true>(M, MS, sc, scd, sfd, K, st, err, a, G * blockIdx.y);
+    if (a < M.N) walks = quad_stream_pops<G, false>(M, MS, sc, scd, K, st, err, a, G * blockIdx.y);
     // one atomic per warp (all lanes here: blocks of whole warps)
     const unsigned wsum = __reduce_add_sync(0xffffffffu, walks);
     if (stats && (threadIdx.x & 31u) == 0u && wsum) atomicAdd(stats, (unsigned long long)wsum);
 }
 
-// The deviation forms in two passes, as on triangles: kq_fast settles the
+// The propagation in two passes, as on triangles: kq_fast settles the
 // populations whose previous-step element passes the certified FP32 test
-// (one thread per population, grid y = direction) and lists the others;
-// kq_slow runs the exact path over the list, spread over all blocks, so
-// that the walks do not hold up the warps of settled populations.
-template <class S, class A>
-__global__ void __launch_bounds__(128) kq_fast(QuadDev M, MapStatic MS, MapScalarsF sfd, KinParams<A> K,
-                                               StateDev<S> st)
+// (grid y: 9 / G direction groups, G directions per thread) and lists the
+// others; kq_slow runs the exact path over the list, spread over all blocks,
+// so that the walks do not hold up the warps of settled populations.  TR: the
+// map is a translation (no map, plunge).
+template <class S, class A, int G, bool TR>
+__global__ void __launch_bounds__(128) kq_fast(QuadDev M, MapStatic MS, MapScalars scd, MapScalarsF sfd,
+                                               KinParams<A> K, StateDev<S> st)
 {
+    constexpr bool FP64 = std::is_same<S, double>::value;
     wait_prior_grid();
-    const int a = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
-    int code = 0;
+    const int a = blockIdx.x * blockDim.x + threadIdx.x, i0 = G * blockIdx.y;
+    int code[G];
+#pragma unroll
+    for (int j = 0; j < G; ++j) code[j] = 0;
     if (a < M.N) {
         const float4 Xf = M.Xf[a];
-        FastMap F = fast_map(MS, sfd, a, Xf);
+        FastMap F = TR ? fast_map_translation(sfd, Xf) : fast_map(MS, sfd, a, Xf);
         if (K.flags & (FLAG_LITERAL_VG | FLAG_EXACT_CHAR)) F.ok = false;
-        code = F.ok && quad_fast_pop<S, A>(M, F, Xf, st, a, i) ? 0 : 1;
+        Node64 n;
+        double2 X;
+        int c[G];
+        if constexpr (FP64) {
+            X = M.X[a];
+            n = node64<TR>(MS, scd, a, X, false);
+#pragma unroll
+            for (int j = 0; j < G; ++j) c[j] = st.cache[(i0 + j) * M.N + a];
+        }
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+            const int i = i0 + j;
+            if (i == 0 && M.vzero[a] && !(K.flags & FLAG_SHIFT)) { // c^_0 exactly zero: the node's own value
+                fg_copy(st.str, st.post, 0, a, M.N);
+            } else if constexpr (FP64) {
+                code[j] = F.ok && quad_fast_pop64<TR>(M, F, n, Xf, X, st, a, i, c[j]) ? 0 : 1;
+            } else {
+                code[j] = F.ok && quad_fast_pop<S, A>(M, F, Xf, st, a, i) ? 0 : 1;
+            }
+        }
     }
-    if (__any_sync(0xffffffffu, code != 0)) append_pop(st, a, M.N, i, code);
+    int any = 0;
+#pragma unroll
+    for (int j = 0; j < G; ++j) any |= code[j];
+    if (__any_sync(0xffffffffu, any != 0)) {
+#pragma unroll
+        for (int j = 0; j < G; ++j) append_pop(st, a, M.N, i0 + j, code[j]);
+    }
 }
 
+// The counter: the deviation forms count the populations that the certified
+// test does not settle (the nodes of zero mesh velocity among them), the FP64
+// form all that are located (9 N less those whose c^ is exactly zero).
 template <class S, class A>
-__global__ void __launch_bounds__(128) kq_slow(QuadDev M, MapStatic MS, MapScalars sc, MapScalars scd,
-                                               MapScalarsF sfd, KinParams<A> K, StateDev<S> st, int *err,
-                                               unsigned long long *stats)
+__global__ void __launch_bounds__(128) kq_slow(QuadDev M, MapStatic MS, MapScalars sc, MapScalars scd, KinParams<A> K,
+                                               StateDev<S> st, int *err, unsigned long long *stats)
 {
+    constexpr bool FP64 = std::is_same<S, double>::value;
     wait_prior_grid();
     __shared__ unsigned pre[NQ + 1];
     if (threadIdx.x == 0) work_prefix(st.wcount, pre);
     __syncthreads();
     const unsigned n = pre[NQ];
-    if (stats && blockIdx.x == 0 && threadIdx.x == 0 && n) atomicAdd(stats, (unsigned long long)n);
+    if (stats && blockIdx.x == 0 && threadIdx.x == 0) {
+        const unsigned nz = K.flags & FLAG_SHIFT ? 0u : (unsigned)M.nvzero;
+        atomicAdd(stats, FP64 ? (unsigned long long)NQ * M.N - nz : (unsigned long long)n + nz);
+    }
     for (unsigned w = spread_first(); w < n; w += spread_stride()) {
         const int code = work_at(st.work, M.N, pre, w);
-        quad_stream_pops<1, false>(M, MS, sc, scd, sfd, K, st, err, code / NQ, code % NQ);
+        const unsigned walks = quad_stream_pops<1, true>(M, MS, sc, scd, K, st, err, code / NQ, code % NQ);
+        if (FP64 && stats && !walks) atomicAdd(stats, ~0ull); // c^ exactly zero: one less
     }
 }
 
-// Directions per thread of kq_stream (the FP64 form): one per population,
+// Directions per thread of kq_stream (the FP64 form where no FP32
+// certificate covers the departure point): one per population,
 // the most threads to hide the walks' dependent loads (3.90 ms per launch
 // at 150k nodes, against 4.00 at three and 4.12 at nine).
 #ifndef ALELB_QUAD_G
@@ -265,30 +318,30 @@ __global__ void __launch_bounds__(256) kq_deriv1(QuadDev M, MapStatic MS, MapSca
     wait_prior_grid();
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= M.N) return;
-    if (!std::is_same<S, double>::value) {
+    if constexpr (!std::is_same<S, double>::value) {
         const FastMap F = fast_map(MS, sf, a, M.Xf[a]);
         float KX, KY;
-        quad_grad_f32(M, a, st.Qx, KX, KY);
+        quad_owner_grad(M, a, st.Qx, KX, KY);
         const float dQx = F.A11 * KX + F.A21 * KY; // d_x Q'_xxx
-        quad_grad_f32(M, a, st.Qy, KX, KY);
+        quad_owner_grad(M, a, st.Qy, KX, KY);
         const float dQy = F.A12 * KX + F.A22 * KY; // d_y Q'_yyy
         const float m = (float)st.mrt[a];
         st.Dx[a] = (fld_t<S>)(m * dQx);
         st.Dy[a] = (fld_t<S>)(m * dQy);
-        return;
+    } else {
+        const double2 Xa = M.X[a];
+        double xX, xY, yX, yY, Vx, Vy, a11, a12, a21, a22;
+        map_node(MS, sc, a, Xa.x, Xa.y, xX, xY, yX, yY, Vx, Vy);
+        metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
+        double KX, KY;
+        quad_owner_grad(M, a, (const double *)st.Qx, KX, KY);
+        const double dQx = a11 * KX + a21 * KY;
+        quad_owner_grad(M, a, (const double *)st.Qy, KX, KY);
+        const double dQy = a12 * KX + a22 * KY;
+        const double m = (double)st.mrt[a];
+        st.Dx[a] = (fld_t<S>)(m * dQx);
+        st.Dy[a] = (fld_t<S>)(m * dQy);
     }
-    const double2 Xa = M.X[a];
-    double xX, xY, yX, yY, Vx, Vy, a11, a12, a21, a22;
-    map_node(MS, sc, a, Xa.x, Xa.y, xX, xY, yX, yY, Vx, Vy);
-    metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
-    double KX, KY;
-    quad_grad(M, M.owner[a], st.Qx, true, KX, KY);
-    const double dQx = a11 * KX + a21 * KY;
-    quad_grad(M, M.owner[a], st.Qy, true, KX, KY);
-    const double dQy = a12 * KX + a22 * KY;
-    const double m = (double)st.mrt[a];
-    st.Dx[a] = (fld_t<S>)(m * dQx);
-    st.Dy[a] = (fld_t<S>)(m * dQy);
 }
 
 // X_a = -d_a D_a in the owner element, then the collision (Eqs. feqn, geqn).
@@ -301,22 +354,24 @@ __global__ void __launch_bounds__(128) kq_collide(QuadDev M, MapStatic MS, MapSc
     if (a >= M.N) return;
     const int N = M.N;
     A Xx = 0, Xy = 0;
-    if (!std::is_same<S, double>::value && !(K.flags & FLAG_PHI_OFF)) {
-        const FastMap F = fast_map(MS, sf, a, M.Xf[a]);
-        float KX, KY;
-        quad_grad_f32(M, a, st.Dx, KX, KY);
-        Xx = (A)(-(F.A11 * KX + F.A21 * KY));
-        quad_grad_f32(M, a, st.Dy, KX, KY);
-        Xy = (A)(-(F.A12 * KX + F.A22 * KY));
+    if constexpr (!std::is_same<S, double>::value) {
+        if (!(K.flags & FLAG_PHI_OFF)) {
+            const FastMap F = fast_map(MS, sf, a, M.Xf[a]);
+            float KX, KY;
+            quad_owner_grad(M, a, st.Dx, KX, KY);
+            Xx = (A)(-(F.A11 * KX + F.A21 * KY));
+            quad_owner_grad(M, a, st.Dy, KX, KY);
+            Xy = (A)(-(F.A12 * KX + F.A22 * KY));
+        }
     } else if (!(K.flags & FLAG_PHI_OFF)) {
         const double2 Xa = M.X[a];
         double xX, xY, yX, yY, Vx, Vy, a11, a12, a21, a22;
         map_node(MS, sc, a, Xa.x, Xa.y, xX, xY, yX, yY, Vx, Vy);
         metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
         double KX, KY;
-        quad_grad(M, M.owner[a], st.Dx, true, KX, KY);
+        quad_owner_grad(M, a, (const double *)st.Dx, KX, KY);
         Xx = (A)(-(a11 * KX + a21 * KY));
-        quad_grad(M, M.owner[a], st.Dy, true, KX, KY);
+        quad_owner_grad(M, a, (const double *)st.Dy, KX, KY);
         Xy = (A)(-(a12 * KX + a22 * KY));
     }
     A f[NQ], g[NQ];
@@ -449,6 +504,10 @@ alelb_status quad_mesh_upload(alelb_mesh *m)
     D.evf = B.put(Q.evf, st);
     D.bdist = B.put(Q.bdist, st);
     D.ownJf = B.put(Q.ownJf, st);
+    D.ownJd = B.put(Q.ownJd, st);
+    D.ebd = B.put(Q.ebd, st);
+    D.vzero = B.put(Q.vzero, st);
+    D.nvzero = (int)std::count(Q.vzero.begin(), Q.vzero.end(), (uint8_t)1);
     m->d_wedges = B.put(Q.wedges, st);
     m->d_n2o = B.put(T.node_new2old, st);
     m->nw = (int)Q.wedges.size();
@@ -475,13 +534,30 @@ cudaError_t quad_launch(alelb_solver *s, int kernel, const MapScalars &sc, const
         case KT_STREAM: {
             constexpr int G = ALELB_QUAD_G;
             launch_pdl(kq_stream<S, A, G>, dim3((N + 127) / 128, NQ / G), dim3(128), s->stream, m->qdev, m->mst, sc,
-                       scd, to_f32(scd, m->T), K, st, s->d_err, s->d_stats);
+                       scd, K, st, s->d_err, s->d_stats);
             break;
         }
-        case KT_FAST:
-            launch_pdl(kq_fast<S, A>, dim3((N + 127) / 128, NQ), dim3(128), s->stream, m->qdev, m->mst,
-                       to_f32(scd, m->T), K, st);
+        case KT_FAST: {
+            const MapScalarsF sfd = to_f32(scd, m->T);
+            const bool tr = m->T.mkind == MK_NONE || m->T.mkind == MK_PLUNGE;
+            const dim3 gb(128), g1((N + 127) / 128, NQ), g3(g1.x, NQ / 3);
+            if (tr) {
+                launch_pdl(kq_fast<S, A, 1, true>, g1, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st);
+                break;
+            }
+            if constexpr (std::is_same<S, double>::value) {
+                // FP64: one map evaluation for three directions from 8k nodes
+                // on (239k blended: 427 us against 539 at one and 446 at nine
+                // per thread; 160k box 280, 318, 326; 24k 54, 62, 80), one per
+                // direction below (1k box: 13, 24, 58 us)
+                if (N >= FAST64_G3_NODES) {
+                    launch_pdl(kq_fast<S, A, 3, false>, g3, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st);
+                    break;
+                }
+            }
+            launch_pdl(kq_fast<S, A, 1, false>, g1, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st);
             break;
+        }
         case KT_SLOW: {
             // every block resident at once (the list spread over all of them)
             static const int per_sm = [] {
@@ -489,8 +565,8 @@ cudaError_t quad_launch(alelb_solver *s, int kernel, const MapScalars &sc, const
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kq_slow<S, A>, 128, 0);
                 return v > 0 ? v : 1;
             }();
-            launch_pdl(kq_slow<S, A>, dim3(per_sm * s->n_sm), dim3(128), s->stream, m->qdev, m->mst, sc, scd,
-                       to_f32(scd, m->T), K, st, s->d_err, s->d_stats);
+            launch_pdl(kq_slow<S, A>, dim3(per_sm * s->n_sm), dim3(128), s->stream, m->qdev, m->mst, sc, scd, K, st,
+                       s->d_err, s->d_stats);
             break;
         }
         case KT_MOMENTS:

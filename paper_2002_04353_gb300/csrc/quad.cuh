@@ -11,9 +11,9 @@
 //
 // The exact path: the FP64 departure point, exact orientation signs for the
 // walk and the tie rules, Newton in the interpolation's arithmetic; the
-// populations are stored and interpolated in the solver's precision.  The
-// deviation forms settle most populations before it with a certified FP32
-// test of the previous-step element (quad_fast_decide).
+// populations are stored and interpolated in the solver's precision.  A
+// certified FP32 test of the previous-step element settles most populations
+// before it (quad_fast_decide).
 #pragma once
 #include "geom.cuh"
 
@@ -126,6 +126,10 @@ struct QuadDev {
     const float4 *evf;     // [4E] corners, FP32 hi + lo
     const float *bdist;    // [N] lower bound of the distance to the nearest boundary edge
     const float4 *ownJf;   // [N] owner element's J^{-1} at the node, FP32
+    const double2 *ownJd;  // [2N] the same in FP64 (grad xi, grad eta)
+    const double2 *ebd;    // [4E] bilinear map: x = b0 + b1 xi + b2 eta + b3 xi eta
+    const uint8_t *vzero;  // [N] 1: mesh velocity exactly zero at all times
+    int nvzero;            // number of those nodes
 };
 
 // The four corners of element e shifted by (sx, sy) periods.
@@ -370,6 +374,94 @@ ALELB_HD __forceinline__ bool quad_local(const QuadDev &M, int e, int sx, int sy
     return quad_newton_t<A>(c, A(1e-5), A(1e-4), xi, eta); // FP32: converged near 1e-7
 }
 
+// Local coordinates of p in element e for the FP64 form: Newton in FP32 on
+// the bilinear map x = b0 + b1 xi + b2 eta + b3 xi eta, then two corrections
+// with the residual in FP64 and the FP32 inverse Jacobian.  A correction
+// leaves about 2^-20 of the error it finds (2^-20 after the FP32 part), so
+// two of them end at the rounding of the residual; each costs 13 operations
+// of the FP64 pipe, against about 60 for a Newton step in FP64.  The rounding
+// of every operation is pinned, so the result is the same in every kernel.
+// false: the corrections did not settle (the last one above 1e-9).
+__device__ __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, int sy, double px, double py,
+                                             double &xi, double &eta)
+{
+    double2 b0 = M.ebd[4 * e];
+    const double2 b1 = M.ebd[4 * e + 1], b2 = M.ebd[4 * e + 2], b3 = M.ebd[4 * e + 3];
+    if (sx) b0.x = da(b0.x, sx * M.Lx);
+    if (sy) b0.y = da(b0.y, sy * M.Ly);
+    const double dx = ds(px, b0.x), dy = ds(py, b0.y);
+    const float fx = (float)dx, fy = (float)dy;
+    const float b1x = (float)b1.x, b1y = (float)b1.y, b2x = (float)b2.x, b2y = (float)b2.y, b3x = (float)b3.x,
+                b3y = (float)b3.y;
+    float u = 0.f, v = 0.f, i11 = 0.f, i12 = 0.f, i21 = 0.f, i22 = 0.f;
+    const auto inverse = [&]() { // J^{-1} at (u, v)
+        const float j11 = __fmaf_rn(b3x, v, b1x), j12 = __fmaf_rn(b3x, u, b2x);
+        const float j21 = __fmaf_rn(b3y, v, b1y), j22 = __fmaf_rn(b3y, u, b2y);
+        const float inv = __frcp_rn(__fmaf_rn(j11, j22, -__fmul_rn(j12, j21)));
+        i11 = __fmul_rn(j22, inv);
+        i12 = -__fmul_rn(j12, inv);
+        i21 = -__fmul_rn(j21, inv);
+        i22 = __fmul_rn(j11, inv);
+    };
+#pragma unroll 1
+    for (int it = 0; it < QUAD_NEWTON_ITERS; ++it) {
+        inverse();
+        const float uv = __fmul_rn(u, v);
+        const float rx = __fsub_rn(fx, __fmaf_rn(b3x, uv, __fmaf_rn(b2x, v, __fmul_rn(b1x, u))));
+        const float ry = __fsub_rn(fy, __fmaf_rn(b3y, uv, __fmaf_rn(b2y, v, __fmul_rn(b1y, u))));
+        const float du = __fmaf_rn(i11, rx, __fmul_rn(i12, ry)), dv = __fmaf_rn(i21, rx, __fmul_rn(i22, ry));
+        u = __fadd_rn(u, du);
+        v = __fadd_rn(v, dv);
+        if (fabsf(du) + fabsf(dv) < 1e-4f) break; // the next step would be below the FP32 rounding
+    }
+    inverse();
+    xi = (double)u;
+    eta = (double)v;
+    float du = 0.f, dv = 0.f;
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+        const double q = dm(xi, eta);
+        const float rx = (float)ds(dx, dfma(b3.x, q, dfma(b2.x, eta, dm(b1.x, xi))));
+        const float ry = (float)ds(dy, dfma(b3.y, q, dfma(b2.y, eta, dm(b1.y, xi))));
+        du = __fmaf_rn(i11, rx, __fmul_rn(i12, ry));
+        dv = __fmaf_rn(i21, rx, __fmul_rn(i22, ry));
+        xi = da(xi, (double)du);
+        eta = da(eta, (double)dv);
+    }
+    return fabsf(du) <= 1e-9f && fabsf(dv) <= 1e-9f;
+}
+
+// The pair (f_i, g_i) of the FP64 form interpolated at (xi, eta) of element
+// e: the nine shape functions are products of one-dimensional ones, so three
+// sums along xi and one along eta (24 operations of the FP64 pipe for the two
+// fields, against 27 for nine weights and their sums).
+__device__ __forceinline__ void quad_interp64(const QuadDev &M, const double *post, int N, int i, int e, double xi,
+                                              double eta, double &f, double &g)
+{
+    int nb[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) nb[k] = M.conn[9 * e + k];
+    const double hx = dm(0.5, xi), hy = dm(0.5, eta);
+    const double lx[3] = {dm(hx, ds(xi, 1.0)), dfma(-xi, xi, 1.0), dm(hx, da(xi, 1.0))};
+    const double ly[3] = {dm(hy, ds(eta, 1.0)), dfma(-eta, eta, 1.0), dm(hy, da(eta, 1.0))};
+    constexpr int at[3][3] = {{0, 4, 1}, {7, 8, 5}, {3, 6, 2}}; // local node at (i, j), row j along xi
+    f = 0.0;
+    g = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        double rf = 0.0, rg = 0.0;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int b = nb[at[j][q]];
+            const double fb = post[i * N + b], gb = post[(NQ + i) * N + b];
+            rf = q ? dfma(lx[q], fb, rf) : dm(lx[q], fb);
+            rg = q ? dfma(lx[q], gb, rg) : dm(lx[q], gb);
+        }
+        f = j ? dfma(ly[j], rf, f) : dm(ly[j], rf);
+        g = j ? dfma(ly[j], rg, g) : dm(ly[j], rg);
+    }
+}
+
 // d K / d X at node a in element el = (elem, local): the nine-node
 // derivative (full = true; Eq. FE_Derivative in the owner element) or the
 // derivative of the bilinear interpolant of the corner values alone (full =
@@ -422,26 +514,52 @@ ALELB_HD __forceinline__ int quad_node_at(int i, int j)
     return (int)((0x263587140ull >> (4 * (3 * j + i))) & 15ull);
 }
 
-// FP32 d K / d X at node a in its owner element (Eq. FE_Derivative): at a
-// node the nine shape functions' xi derivatives vanish off the node's eta
-// row and their eta derivatives off its xi column, so each derivative is a
-// three-term sum; dL_m at the node's coordinate t in {-1, 0, 1} is t - 1/2,
-// -2 t, t + 1/2 (exact in FP32).
+// d K / d X at node a in its owner element (Eq. FE_Derivative), in the
+// arithmetic of the form (float, or double for FP64 fields): at a node the
+// nine shape functions' xi derivatives vanish off the node's eta row and
+// their eta derivatives off its xi column, so each derivative is a three-term
+// sum; dL_m at the node's coordinate t in {-1, 0, 1} is t - 1/2, -2 t, t + 1/2
+// (exact).
+template <class S> struct QuadJ;
+template <> struct QuadJ<float> {
+    static __device__ __forceinline__ void get(const QuadDev &M, int a, float J[4])
+    {
+        const float4 v = M.ownJf[a];
+        J[0] = v.x;
+        J[1] = v.y;
+        J[2] = v.z;
+        J[3] = v.w;
+    }
+};
+template <> struct QuadJ<double> {
+    static __device__ __forceinline__ void get(const QuadDev &M, int a, double J[4])
+    {
+        const double2 p = M.ownJd[2 * a], q = M.ownJd[2 * a + 1];
+        J[0] = p.x;
+        J[1] = p.y;
+        J[2] = q.x;
+        J[3] = q.y;
+    }
+};
 template <class S>
-__device__ __forceinline__ void quad_grad_f32(const QuadDev &M, int a, const S *K, float &KX, float &KY)
+__device__ __forceinline__ void quad_owner_grad(const QuadDev &M, int a, const S *K, S &KX, S &KY)
 {
     const int2 ow = M.owner[a];
     const int e = ow.x, l = ow.y;
     const int li = quad_ix(l), lj = quad_iy(l);
-    const float tx = (float)(li - 1), ty = (float)(lj - 1);
     const int *cn = M.conn + 9 * e;
-    const float sxi = (tx - 0.5f) * (float)K[cn[quad_node_at(0, lj)]] + (-2.0f * tx) * (float)K[cn[quad_node_at(1, lj)]] +
-                      (tx + 0.5f) * (float)K[cn[quad_node_at(2, lj)]];
-    const float seta = (ty - 0.5f) * (float)K[cn[quad_node_at(li, 0)]] + (-2.0f * ty) * (float)K[cn[quad_node_at(li, 1)]] +
-                       (ty + 0.5f) * (float)K[cn[quad_node_at(li, 2)]];
-    const float4 J = M.ownJf[a];
-    KX = sxi * J.x + seta * J.z;
-    KY = sxi * J.y + seta * J.w;
+    // the three weights by selection (t = li - 1): no FP64 conversion
+    const auto w0 = [](int c) { return c == 0 ? S(-1.5) : c == 1 ? S(-0.5) : S(0.5); };
+    const auto w1 = [](int c) { return c == 0 ? S(2) : c == 1 ? S(0) : S(-2); };
+    const auto w2 = [](int c) { return c == 0 ? S(-0.5) : c == 1 ? S(0.5) : S(1.5); };
+    const S sxi = w0(li) * K[cn[quad_node_at(0, lj)]] + w1(li) * K[cn[quad_node_at(1, lj)]] +
+                  w2(li) * K[cn[quad_node_at(2, lj)]];
+    const S seta = w0(lj) * K[cn[quad_node_at(li, 0)]] + w1(lj) * K[cn[quad_node_at(li, 1)]] +
+                   w2(lj) * K[cn[quad_node_at(li, 2)]];
+    S J[4];
+    QuadJ<S>::get(M, a, J);
+    KX = sxi * J[0] + seta * J[2];
+    KY = sxi * J[1] + seta * J[3];
 }
 
 } // namespace alelb

@@ -29,6 +29,12 @@ struct QuadTables {
     // the FP32 derivative passes: J^{-1} of the owner element's bilinear map
     // at the node, (d xi/dX, d xi/dY, d eta/dX, d eta/dY)
     std::vector<float4> ownJf; // [N]
+    // the FP64 form: the same J^{-1} in FP64 (rows grad xi, grad eta), the
+    // bilinear map's coefficients of each element, and the nodes whose mesh
+    // velocity is zero at all times
+    std::vector<double2> ownJd; // [2N]
+    std::vector<double2> ebd;   // [4E] b0, b1, b2, b3: x = b0 + b1 xi + b2 eta + b3 xi eta
+    std::vector<uint8_t> vzero; // [N]
 };
 
 // Local coordinates of p in the quadrilateral with corners w (x, y pairs),
@@ -343,6 +349,7 @@ inline alelb_status build_quad_tables(const alelb_mesh_desc *d, HostTables &T, Q
     Q.evf.resize((size_t)4 * E);
     for (size_t k = 0; k < (size_t)4 * E; ++k) Q.evf[k] = split(Q.ev[k]);
     Q.ownJf.resize(N);
+    Q.ownJd.resize((size_t)2 * N);
     for (int a = 0; a < N; ++a) {
         const int e = Q.owner[a].x, l = Q.owner[a].y;
         double w[8], x, y, J[4];
@@ -353,6 +360,24 @@ inline alelb_status build_quad_tables(const alelb_mesh_desc *d, HostTables &T, Q
         quad_bilinear(w, quad_ix(l) - 1.0, quad_iy(l) - 1.0, x, y, J);
         const double det = J[0] * J[3] - J[2] * J[1];
         Q.ownJf[a] = make_float4((float)(J[3] / det), (float)(-J[1] / det), (float)(-J[2] / det), (float)(J[0] / det));
+        Q.ownJd[2 * a] = make_double2(J[3] / det, -J[1] / det);
+        Q.ownJd[2 * a + 1] = make_double2(-J[2] / det, J[0] / det);
+    }
+    Q.ebd.resize((size_t)4 * E);
+    for (int e = 0; e < E; ++e) {
+        const double2 *v = Q.ev.data() + (size_t)4 * e;
+        // differences of the corners (exact for nearby coordinates), then halves and sums
+        auto coef = [](double a, double b, double c, double d, double o[4]) {
+            const double u = b - a, w = c - d; // along the lower and the upper edge
+            o[0] = 0.25 * (((a + b) + c) + d);
+            o[1] = 0.25 * (u + w);
+            o[2] = 0.25 * ((d - a) + (c - b));
+            o[3] = 0.25 * (w - u);
+        };
+        double bx[4], by[4];
+        coef(v[0].x, v[1].x, v[2].x, v[3].x, bx);
+        coef(v[0].y, v[1].y, v[2].y, v[3].y, by);
+        for (int k = 0; k < 4; ++k) Q.ebd[(size_t)4 * e + k] = make_double2(bx[k], by[k]);
     }
     // lower bound of every node's distance to the nearest boundary edge,
     // capped at DCAP (zero on periodic meshes with boundaries: those always
@@ -396,6 +421,8 @@ inline alelb_status build_quad_tables(const alelb_mesh_desc *d, HostTables &T, Q
         }
     }
     T.ms = static_map_factors(T.mkind, T.mp, T.X);
+    Q.vzero.assign(N, 0);
+    for (int a = 0; a < N; ++a) Q.vzero[a] = (uint8_t)(T.mkind == MK_NONE || (T.mkind == MK_BLENDED && T.ms[a] == 0.0));
     T.msf.resize(T.ms.size());
     for (size_t k = 0; k < T.ms.size(); ++k) T.msf[k] = (float)T.ms[k];
     T.n_wall_nodes = (int)Q.probe_e.size();

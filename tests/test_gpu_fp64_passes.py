@@ -11,14 +11,15 @@ from paper_2002_04353_gb300 import inputs as I
 pytestmark = pytest.mark.gpu
 
 
-def _case(kind, n):
+def _case(kind, n, elem):
     if kind == "box":
-        return I.uniform_flow_case(n=n, L=2.0 * n, period_steps=40.0)
+        return I.uniform_flow_case(n=n, L=2.0 * n, period_steps=40.0, elem=elem)
     ni, nj = I.omesh_size_for(n)
     if kind == "plunge":
-        c = I.plunge_case(ni=ni, nj=nj)
+        c = I.plunge_case(ni=ni, nj=nj, elem=elem)
     else:
-        c = I.pitch_case(ni=ni, nj=nj, Ma=0.3, blended=kind == "blended", plunge_frac=0.0 if kind == "blended" else 0.05)
+        c = I.pitch_case(ni=ni, nj=nj, Ma=0.3, blended=kind == "blended", plunge_frac=0.0 if kind == "blended" else 0.05,
+                         elem=elem)
     return dataclasses.replace(c, flow=dataclasses.replace(c.flow, flags=256))
 
 
@@ -35,9 +36,10 @@ def _start(case, seed):
 
 @pytest.mark.parametrize("kind,n", [("box", 7), ("box", 46), ("box", 130), ("plunge", 9000), ("pitch", 6000), ("blended", 21000),
                                     ("blended", 66000)])
-def test_values_do_not_depend_on_the_cache(kind, n):
+@pytest.mark.parametrize("elem", ["p2", "q2"])
+def test_values_do_not_depend_on_the_cache(kind, n, elem):
     from paper_2002_04353_gb300 import alelb
-    case = _case(kind, n)
+    case = _case(kind, n, elem)
     warm = _start(case, 1)
     warm.lb_step(3)
     f, g = warm.get_pops()
@@ -53,9 +55,10 @@ def test_values_do_not_depend_on_the_cache(kind, n):
 
 
 @pytest.mark.parametrize("kind,n", [("box", 45), ("box", 46), ("box", 129), ("pitch", 8000)])
-def test_against_the_oracle(kind, n):
+@pytest.mark.parametrize("elem", ["p2", "q2"])
+def test_against_the_oracle(kind, n, elem):
     import oracle as O
-    case = _case(kind, n)
+    case = _case(kind, n, elem)
     s = _start(case, 2)
     f, g = s.get_pops()
     m = s.moments()
