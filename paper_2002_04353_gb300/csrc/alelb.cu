@@ -77,7 +77,7 @@ alelb_status check_sticky(alelb_solver *s)
 
 namespace {
 
-template <class S> void put_state(DevBuf &b, StateDev<S> &s, int N, cudaError_t &st)
+template <class S> void put_state(DevBuf &b, StateDev<S> &s, int N, int mkind, cudaError_t &st)
 {
     using P = pop_t<S>;
     using F = fld_t<S>;
@@ -97,6 +97,7 @@ template <class S> void put_state(DevBuf &b, StateDev<S> &s, int N, cudaError_t 
     s.work = b.alloc<int>((size_t)(SEG_PENDING + 1) * N, st);
     s.wcount = b.alloc<unsigned>(SEG_PENDING + 1, st);
     if (st == cudaSuccess) st = cudaMemset(s.wcount, 0, (SEG_PENDING + 1) * sizeof(unsigned));
+    s.met = std::is_same<S, double>::value && !uniform_metric(mkind) ? b.alloc<double2>((size_t)2 * N, st) : nullptr;
     s.wmask = b.alloc<unsigned>(N, st);
     if (st == cudaSuccess) st = cudaMemset(s.wmask, 0, (size_t)N * sizeof(unsigned));
 }
@@ -456,8 +457,12 @@ cudaEvent_t get_event(alelb_solver *s)
 
 
 template <class S, class A>
-cudaError_t launch_step(alelb_solver *s, StateDev<S> &st, KinParams<A> &K, const MapScalars &sc_in)
+cudaError_t launch_step(alelb_solver *s, const StateDev<S> &st0, KinParams<A> &K, const MapScalars &sc_in)
 {
+    StateDev<S> st = st0;
+    // the propagation leaves the metrics only where it evaluates the map of
+    // the arrival time
+    if (s->flags & (ALELB_FLAG_LITERAL_VG | ALELB_FLAG_EXACT_CHAR | ALELB_FLAG_MIDPOINT)) st.met = nullptr;
     alelb_mesh *m = s->mesh;
     const MapScalars sc = solver_map(s, sc_in);
     const int N = m->T.N;
@@ -504,6 +509,7 @@ cudaError_t launch_step(alelb_solver *s, StateDev<S> &st, KinParams<A> &K, const
         seq[ns++] = KT_MOMENTS;
     } else {
         seq[ns++] = KT_STREAM;
+        seq[ns++] = KT_MOMENTS;
     }
     if (phi) seq[ns++] = KT_DERIV1;
     seq[ns++] = KT_COLLIDE;
@@ -572,20 +578,11 @@ cudaError_t launch_step(alelb_solver *s, StateDev<S> &st, KinParams<A> &K, const
             launch_pdl(k_moments<S, A>, dim3((N + 255) / 256), dim3(256), s->stream, K, st, N, s->d_err);
             break;
         case KT_DERIV1:
-            if (fast)
-                launch_pdl(k_deriv1<S, A, true>, dim3((N + 255) / 256), dim3(256), s->stream, m->dev, m->mst, sc,
-                           sf, st);
-            else
-                launch_pdl(k_deriv1<S, A, false>, dim3((N + 255) / 256), dim3(256), s->stream, m->dev, m->mst, sc,
-                           sf, st);
+            launch_pdl(k_deriv1<S, A>, dim3((N + 255) / 256), dim3(256), s->stream, m->dev, m->mst, sc, sf, st);
             break;
         default:
-            if (fast)
-                launch_pdl(k_collide<S, A, true>, dim3((N + 127) / 128), dim3(128), s->stream, m->dev, m->mst, sc,
-                           sf, K, st, s->d_err);
-            else
-                launch_pdl(k_collide<S, A, false>, dim3((N + 127) / 128), dim3(128), s->stream, m->dev, m->mst,
-                           sc, sf, K, st, s->d_err);
+            launch_pdl(k_collide<S, A>, dim3((N + 127) / 128), dim3(128), s->stream, m->dev, m->mst, sc, sf, K, st,
+                       s->d_err);
         }
         if (s->prof) {
             cudaEventRecord(eb, s->stream);
@@ -601,6 +598,8 @@ template <class A> void fill_kin(alelb_solver *s, KinParams<A> &K)
     K.Cp = (A)s->Cp;
     K.mu = (A)s->mu;
     K.Pr = (A)s->Pr;
+    K.iCv = (A)(1.0 / s->Cv);
+    K.iPr = (A)(1.0 / s->Pr);
     double r = 0, jx = 0, jy = 0, pxx = 0, pxy = 0, pyy = 0, e2 = 0;
     for (int i = 0; i < NQ; ++i) {
         const double fr = s->consts[i];
@@ -681,7 +680,7 @@ extern "C" alelb_status alelb_lb_init(alelb_mesh *m, const alelb_params *p, alel
             cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && nsm > 0)
             s->n_sm = nsm;
     }
-    with_state(s, [&](auto &sx, auto &) { put_state(s->buf, sx, N, st); });
+    with_state(s, [&](auto &sx, auto &) { put_state(s->buf, sx, N, m->T.mkind, st); });
     s->d_consts = s->buf.alloc<double>(4 * NQ, st);
     s->d_scratch = s->buf.alloc<double>((size_t)22 * N, st);
     s->d_err = s->buf.alloc<int>(1, st);
@@ -1275,6 +1274,8 @@ extern "C" alelb_status alelb_lb_step_noalloc(alelb_mesh *m, const alelb_params 
     K.Cp = K.Cv + 1.0;
     K.mu = p->mu;
     K.Pr = p->Pr;
+    K.iCv = 1.0 / K.Cv;
+    K.iPr = 1.0 / K.Pr;
     K.rho_ref = 0.0;
     K.E2_ref = 0.0;
     for (int i = 0; i < NQ; ++i) {
@@ -1290,10 +1291,10 @@ extern "C" alelb_status alelb_lb_step_noalloc(alelb_mesh *m, const alelb_params 
         : (p->flags & ALELB_FLAG_MIDPOINT) ? with_shift(map_scalars(m->T.mkind, m->T.mp, t + 0.5), p->shift)
                                            : sc;
     k_stream<double, double><<<(N + 127) / 128, 128, 0, stream>>>(m->dev, m->mst, sc, scd, K, sd, err, nullptr);
+    k_moments<double, double><<<(N + 255) / 256, 256, 0, stream>>>(K, sd, N, err);
     if (!(p->flags & (ALELB_FLAG_PHI_OFF | ALELB_FLAG_COLLIDE_OFF)))
-        k_deriv1<double, double, false><<<(N + 255) / 256, 256, 0, stream>>>(m->dev, m->mst, sc, to_f32(sc, m->T), sd);
-    k_collide<double, double, false><<<(N + 127) / 128, 128, 0, stream>>>(m->dev, m->mst, sc, to_f32(sc, m->T), K,
-                                                                        sd, err);
+        k_deriv1<double, double><<<(N + 255) / 256, 256, 0, stream>>>(m->dev, m->mst, sc, to_f32(sc, m->T), sd);
+    k_collide<double, double><<<(N + 127) / 128, 128, 0, stream>>>(m->dev, m->mst, sc, to_f32(sc, m->T), K, sd, err);
     int herr = 0;
     st = cudaGetLastError();
     if (st == cudaSuccess) st = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, stream);

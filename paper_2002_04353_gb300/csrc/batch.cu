@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(T *NQ / G) kb_fast_fused(const CaseDev<float, 
     }
 }
 
-template <class S, class A, bool FAST>
+template <class S, class A>
 __global__ void __launch_bounds__(256) kb_deriv1(const CaseDev<S, A> *__restrict__ cases,
                                                  const int *__restrict__ off, int B,
                                                  const MapScalars *__restrict__ sc,
@@ -329,10 +329,10 @@ __global__ void __launch_bounds__(256) kb_deriv1(const CaseDev<S, A> *__restrict
     __syncthreads();
     const CaseDev<S, A> &C = sh.C();
     const int a = (blockIdx.x - __ldg(off + c)) * blockDim.x + threadIdx.x;
-    if (a < C.M.N) deriv1_node<S, A, FAST>(C.M, C.MS, sh.SC(), sh.SF(), C.st, a);
+    if (a < C.M.N) deriv1_node<S, A>(C.M, C.MS, sh.SC(), sh.SF(), C.st, a);
 }
 
-template <class S, class A, bool FAST>
+template <class S, class A>
 __global__ void __launch_bounds__(256) kb_collide(const CaseDev<S, A> *__restrict__ cases,
                                                   const int *__restrict__ off, int B,
                                                   const MapScalars *__restrict__ sc,
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(256) kb_collide(const CaseDev<S, A> *__restric
     __syncthreads();
     const CaseDev<S, A> &C = sh.C();
     const int a = (blockIdx.x - __ldg(off + c)) * blockDim.x + threadIdx.x;
-    if (a < C.M.N) collide_at<S, A, FAST>(C.M, C.MS, sh.SC(), sh.SF(), C.K, C.st, C.err, a);
+    if (a < C.M.N) collide_at<S, A>(C.M, C.MS, sh.SC(), sh.SF(), C.K, C.st, C.err, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -570,7 +570,6 @@ __global__ void __launch_bounds__(128) kb_persistent(const CaseDev<S, A> *__rest
                                                      const MapScalarsF *__restrict__ sfs, int K, GridSync g)
 {
     constexpr int NS = NQ + 1;
-    constexpr bool FAST = !std::is_same<S, double>::value;
     __shared__ SharedCase<S, A> sh;
     __shared__ unsigned pre[BATCH_MAX * NS + 1];
     const int tiles = __ldg(off + B);
@@ -649,11 +648,11 @@ __global__ void __launch_bounds__(128) kb_persistent(const CaseDev<S, A> *__rest
         });
         if (!grid_barrier(g, cases, B)) return;
         tiles_loop(k, [&](const CaseDev<S, A> &C, const MapScalars &SC, const MapScalarsF &SF, int a) {
-            if (a < C.M.N) deriv1_node<S, A, FAST>(C.M, C.MS, SC, SF, C.st, a);
+            if (a < C.M.N) deriv1_node<S, A>(C.M, C.MS, SC, SF, C.st, a);
         });
         if (!grid_barrier(g, cases, B)) return;
         tiles_loop(k, [&](const CaseDev<S, A> &C, const MapScalars &SC, const MapScalarsF &SF, int a) {
-            if (a < C.M.N) collide_at<S, A, FAST>(C.M, C.MS, SC, SF, C.K, C.st, C.err, a);
+            if (a < C.M.N) collide_at<S, A>(C.M, C.MS, SC, SF, C.K, C.st, C.err, a);
         });
         if (!grid_barrier(g, cases, B)) return;
     }
@@ -884,13 +883,13 @@ void launch_phase(alelb_batch *b, const Part &P, int kt, int bs, int grid, int k
         if (fast)
             launch_after(P.pdl, kb_deriv1_staged, dim3(tiles), dim3(bs), P.stream,
                        reinterpret_cast<const CaseDev<float, float> *>(cases), off, B, sf, (int)stage);
-        else launch_after(P.pdl, kb_deriv1<S, A, false>, dim3(tiles), dim3(bs), P.stream, cases, off, B, sc, sf);
+        else launch_after(P.pdl, kb_deriv1<S, A>, dim3(tiles), dim3(bs), P.stream, cases, off, B, sc, sf);
         break;
     default:
         if (fast)
             launch_after(P.pdl, kb_collide_staged, dim3(tiles), dim3(bs), P.stream,
                        reinterpret_cast<const CaseDev<float, float> *>(cases), off, B, sf, (int)stage);
-        else launch_after(P.pdl, kb_collide<S, A, false>, dim3(tiles), dim3(bs), P.stream, cases, off, B, sc, sf);
+        else launch_after(P.pdl, kb_collide<S, A>, dim3(tiles), dim3(bs), P.stream, cases, off, B, sc, sf);
     }
 }
 

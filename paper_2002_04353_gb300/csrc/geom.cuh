@@ -34,7 +34,10 @@ struct MapScalars {
     double c, sn, thd; // rotation: cos, sin, angular rate
     double cm;         // cos - 1
     double Ux, Uy;     // lattice shift U: the velocities are c_i + U (zero when unshifted)
+    double A11, A12, A21, A22; // g^{-1,T} of the rigid maps (uniform_metric), the canonical operations on the host
 };
+// Kinds whose metrics do not depend on the node.
+__host__ __device__ constexpr bool uniform_metric(int kind) { return kind != MK_SINE && kind != MK_BLENDED; }
 
 struct MapStatic {
     int kind;
@@ -106,6 +109,15 @@ ALELB_HD __forceinline__ void set_err(int *err, int bit)
 #else
     *err |= bit;
 #endif
+}
+
+// A float as a double by its bits (the FP64 pipe runs conversions at its own
+// low rate): exact for 0 and normal numbers; a subnormal one is not kept.
+__device__ __forceinline__ double f2d_bits(float v)
+{
+    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+    const unsigned hi = m >= 0x00800000u ? (b & 0x80000000u) | ((m >> 3) + 0x38000000u) : 0u;
+    return __hiloint2double((int)hi, (int)(m >= 0x00800000u ? b << 29 : 0u));
 }
 
 // Metrics x_X, x_Y, y_X, y_Y and mesh velocity V_G at a node.

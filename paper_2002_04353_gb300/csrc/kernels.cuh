@@ -12,10 +12,9 @@
 //
 //   k_stream   transformed velocities, departure points, element walk, P2
 //              interpolation of the post-collision populations, Grad-type
-//              missing populations (Sec. IV.A); then moments, Q'_aaa (Eq.
-//              DeviationTerms) and mu/(rho T).  It serves the step that
-//              keeps no state of its own (no element cache) and the departure
-//              points that no FP32 certificate covers.
+//              missing populations (Sec. IV.A); k_moments follows.  It serves
+//              the step that keeps no state of its own (no element cache) and
+//              the departure points that no FP32 certificate covers.
 //
 // One thread per node unless noted.  Populations are stored by direction: FP64 buffers
 // as pop[q * N + node] with q = 0..8 for f and 9..17 for g, the deviation
@@ -153,6 +152,9 @@ template <class S> struct StateDev {
                           // moments the fused batched propagation left to the moments
                           // kernel, at work[10 N + k], k < wcount[10]
     unsigned *wcount;     // [11] entries of each segment
+    double2 *met;         // [2N] FP64 form on a map whose metrics vary: A of each node at the
+                          // arrival time, (A11, A12), (A21, A22), left by the propagation for
+                          // the derivative passes; null: they evaluate the map
     unsigned *wmask;      // [N] directions certified missing at a wall (bits 0-8); set by the
                           // propagation kernel, read by the exact path, cleared by the
                           // moments kernel
@@ -338,9 +340,40 @@ __device__ __forceinline__ Node64 node64(const MapStatic &MS, const MapScalars &
     }
     double xX, xY, yX, yY, Vx, Vy;
     map_node(MS, sc, a, X.x, X.y, xX, xY, yX, yY, Vx, Vy);
-    metric_inverse_T(xX, xY, yX, yY, n.a11, n.a12, n.a21, n.a22);
+    if (uniform_metric(MS.kind)) {
+        n.a11 = sc.A11;
+        n.a12 = sc.A12;
+        n.a21 = sc.A21;
+        n.a22 = sc.A22;
+    } else {
+        metric_inverse_T(xX, xY, yX, yY, n.a11, n.a12, n.a21, n.a22);
+    }
     mesh_velocity_term(n.a11, n.a12, n.a21, n.a22, ds(Vx, sc.Ux), ds(Vy, sc.Uy), literal, n.wx, n.wy);
     return n;
+}
+
+// A = g^{-1,T} of node a at the arrival time, for the derivative passes of
+// the FP64 form: uniform, or as the propagation left it, or from the map.
+__device__ __forceinline__ void metric64(const MapStatic &MS, const MapScalars &sc, const double2 *Xs,
+                                         const StateDev<double> &st, int a, double A[4])
+{
+    if (uniform_metric(MS.kind)) {
+        A[0] = sc.A11;
+        A[1] = sc.A12;
+        A[2] = sc.A21;
+        A[3] = sc.A22;
+    } else if (st.met) {
+        const double2 p = st.met[2 * a], q = st.met[2 * a + 1];
+        A[0] = p.x;
+        A[1] = p.y;
+        A[2] = q.x;
+        A[3] = q.y;
+    } else {
+        const double2 X = Xs[a];
+        double xX, xY, yX, yY, Vx, Vy;
+        map_node(MS, sc, a, X.x, X.y, xX, xY, yX, yY, Vx, Vy);
+        metric_inverse_T(xX, xY, yX, yY, A[0], A[1], A[2], A[3]);
+    }
 }
 
 // a cx + b cy for cx, cy in {-1, 0, 1}: the value of da(dm(a, cx), dm(b, cy))
@@ -413,8 +446,6 @@ __device__ __forceinline__ void stream_plain_node(const MeshDev &M, const MapSta
     double a11 = 0, a12 = 0, a21 = 0, a22 = 0, wx = 0, wy = 0, Vx = 0, Vy = 0;
     int miss = 0, far = 0;
     unsigned walks = 0;
-    // running moments of the streamed populations (deviations)
-    A sfm = 0, jx = 0, jy = 0, sg = 0;
 #pragma unroll 1
     for (int i = 0; i < NQ; ++i) {
         A fi = 0, gi = 0;
@@ -468,10 +499,6 @@ __device__ __forceinline__ void stream_plain_node(const MeshDev &M, const MapSta
             fg_get(st.post, i, src, N, fi, gi);
         }
         fg_put(st.str, i, a, N, fi, gi);
-        sfm += fi;
-        jx += (A)c_cx[i] * fi;
-        jy += (A)c_cy[i] * fi;
-        sg += gi;
     }
     if (stats && walks) atomicAdd(stats, (unsigned long long)walks);
     if (miss) {
@@ -488,24 +515,8 @@ __device__ __forceinline__ void stream_plain_node(const MeshDev &M, const MapSta
             A fi = (far >> i & 1) ? K.finf[i] : fm[i];
             A gi = (far >> i & 1) ? K.ginf[i] : gm[i];
             fg_put(st.str, i, a, N, fi, gi);
-            sfm += fi;
-            jx += (A)c_cx[i] * fi;
-            jy += (A)c_cy[i] * fi;
-            sg += gi;
         }
     }
-    // moments (Sec. IV): rho, u, E, T from the streamed populations
-    A rho = K.rho_ref + sfm;
-    // w = u - U (relative to the lattice shift), u = w + U
-    A rwx = (K.jx_ref + jx) / rho, rwy = (K.jy_ref + jy) / rho;
-    A ux = rwx + K.Ux, uy = rwy + K.Uy;
-    A E = (K.E2_ref + sg) / (A(2) * rho);
-    A T = (E - A(0.5) * (ux * ux + uy * uy)) / K.Cv;
-    if (!(rho > A(0)) || !(T > A(0)) || !isfinite(rho) || !isfinite(T)) atomicOr(err, ERR_NONFINITE);
-    A k3 = A(1) - A(3) * T;
-    st.Qx[a] = (fld_t<S>)(rho * rwx * k3 - rho * rwx * rwx * rwx);
-    st.Qy[a] = (fld_t<S>)(rho * rwy * k3 - rho * rwy * rwy * rwy);
-    st.mrt[a] = (fld_t<S>)(K.mu / (rho * T));
 }
 
 template <class S, class A>
@@ -769,6 +780,10 @@ __device__ __forceinline__ void stream_fast_pops64(const MeshDev &M, const MapSt
     FastMap F = TR ? fast_map_translation(sf, Xf) : fast_map(MS, sf, a, Xf);
     if (K.flags & (FLAG_LITERAL_VG | FLAG_EXACT_CHAR)) F.ok = false;
     const Node64 n = node64<TR>(MS, sc, a, X, false);
+    if (!TR && i0 == 0 && st.met) { // for the derivative passes
+        st.met[2 * a] = make_double2(n.a11, n.a12);
+        st.met[2 * a + 1] = make_double2(n.a21, n.a22);
+    }
 #pragma unroll
     for (int j = 0; j < G; ++j) {
         const int i = i0 + j;
@@ -1065,11 +1080,29 @@ __device__ __forceinline__ void moments_store(const KinParams<A> &K, const State
     st.mrt[a] = (fld_t<S>)(K.mu / (rho * T));
 }
 
+// The FP64 form: the fields themselves are stored too, for the collision
+// (the previous step's were last read by the exact path).
+__device__ __forceinline__ void moments_store(const KinParams<double> &K, const StateDev<double> &st, int *err, int a,
+                                              const double f[NQ], const double g[NQ])
+{
+    double rho, jx, jy, wx, wy, ux, uy, T;
+    fields64(K, f, g, rho, jx, jy, wx, wy, ux, uy, T);
+    if (!(rho > 0.0) || !(T > 0.0) || !isfinite(rho) || !isfinite(T)) atomicOr(err, ERR_NONFINITE);
+    const double k3 = 1.0 - 3.0 * T;
+    st.Qx[a] = jx * (k3 - wx * wx); // rho w = j
+    st.Qy[a] = jy * (k3 - wy * wy);
+    st.mrt[a] = K.mu / (rho * T);
+    st.rho[a] = rho;
+    st.ux[a] = ux;
+    st.uy[a] = uy;
+    st.T[a] = T;
+}
+
 template <class S, class A>
 __device__ __forceinline__ void moments_node(const KinParams<A> &K, const StateDev<S> &st, int N,
                                              int *err, int a)
 {
-    st.wmask[a] = 0u; // used by the exact path of this step
+    if (st.wmask) st.wmask[a] = 0u; // used by the exact path of this step
     A f[NQ], g[NQ];
 #pragma unroll
     for (int i = 0; i < NQ; ++i) {
@@ -1083,7 +1116,7 @@ __global__ void __launch_bounds__(256) k_moments(KinParams<A> K, StateDev<S> st,
 {
     wait_prior_grid();
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a <= NQ) st.wcount[a] = 0u; // the work list has been consumed
+    if (st.wcount && a <= NQ) st.wcount[a] = 0u; // the work list has been consumed
     if (a < N) moments_node(K, st, N, err, a);
 }
 
@@ -1166,6 +1199,48 @@ __device__ __forceinline__ void owner_grad_f32(const MeshDev &M, int a, const S 
     KY = sxi * J.y + seta * J.w;
 }
 
+// d_x K0 and d_y K1 of two node fields at node a in FP64, in its owner
+// element (the divergence terms of both derivative passes): the derivative
+// weights at a node are small integers, formed by integer operations; the
+// element's stored FP64 inverse Jacobian; the node's metrics (metric64).
+// 48 operations of the FP64 pipe, 24 on a translation, against about 135 with
+// the map, the Jacobian and their divisions evaluated per node (k_deriv1 of
+// the 150,400-node plunge: 31 us before).
+__device__ __forceinline__ void owner_div64(const MeshDev &M, const MapStatic &MS, const MapScalars &sc,
+                                            const StateDev<double> &st, int a, const double *K0, const double *K1,
+                                            double &d0, double &d1)
+{
+    const int4 p = M.ostn[2 * a], q = M.ostn[2 * a + 1];
+    const int e = q.z;
+    const double2 j1 = M.ejd[2 * e], j2 = M.ejd[2 * e + 1];
+    const int nb[6] = {p.x, p.y, p.z, p.w, q.x, q.y};
+    float nx[6], ne[6];
+    p2_dN_at_node(q.w, nx, ne);
+    double x0 = 0, e0 = 0, x1 = 0, e1 = 0;
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+        const double v0 = K0[nb[s]], v1 = K1[nb[s]];
+        if (s != 2) { // d N_2 / d xi = 0
+            const double w = f2d_bits(nx[s]);
+            x0 += v0 * w;
+            x1 += v1 * w;
+        }
+        if (s != 1) { // d N_1 / d eta = 0
+            const double w = f2d_bits(ne[s]);
+            e0 += v0 * w;
+            e1 += v1 * w;
+        }
+    }
+    d0 = x0 * j1.x + e0 * j2.x; // d K0 / d X
+    d1 = x1 * j1.y + e1 * j2.y; // d K1 / d Y
+    if (MS.kind == MK_NONE || MS.kind == MK_PLUNGE) return; // A = I
+    double A[4];
+    metric64(MS, sc, M.X, st, a, A);
+    const double d0Y = x0 * j1.y + e0 * j2.y, d1X = x1 * j1.x + e1 * j2.x;
+    d0 = A[0] * d0 + A[2] * d0Y;
+    d1 = A[1] * d1X + A[3] * d1;
+}
+
 // First-order FP32 d K / d X for the wall condition, through the vertices
 // of the node's smallest incident element.
 template <class S>
@@ -1181,12 +1256,12 @@ __device__ __forceinline__ void owner_grad_linear_f32(const MeshDev &M, int a, c
     KY = sxi * J.y + seta * J.w;
 }
 
-template <class S, class A, bool FAST>
+template <class S, class A>
 __device__ __forceinline__ void deriv1_node(const MeshDev &M, const MapStatic &MS,
                                             const MapScalars &sc, const MapScalarsF &sf,
                                             const StateDev<S> &st, int a)
 {
-    if (FAST) {
+    if constexpr (!std::is_same<S, double>::value) {
         const FastMap F = fast_map(MS, sf, a, M.Xf[a]);
         float KX, KY;
         owner_grad_f32(M, a, st.Qx, KX, KY);
@@ -1196,56 +1271,64 @@ __device__ __forceinline__ void deriv1_node(const MeshDev &M, const MapStatic &M
         const float m = (float)st.mrt[a];
         st.Dx[a] = (fld_t<S>)(m * dQx);
         st.Dy[a] = (fld_t<S>)(m * dQy);
-        return;
+    } else {
+        double dQx, dQy;
+        owner_div64(M, MS, sc, st, a, st.Qx, st.Qy, dQx, dQy);
+        const double m = st.mrt[a];
+        st.Dx[a] = m * dQx;
+        st.Dy[a] = m * dQy;
     }
-    const double2 Xa = M.X[a];
-    double xX, xY, yX, yY, Vx, Vy, a11, a12, a21, a22;
-    map_node(MS, sc, a, Xa.x, Xa.y, xX, xY, yX, yY, Vx, Vy);
-    metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
-    double KX, KY;
-    owner_grad(M, a, st.Qx, KX, KY);
-    double dQx = a11 * KX + a21 * KY; // d_x Q'_xxx
-    owner_grad(M, a, st.Qy, KX, KY);
-    double dQy = a12 * KX + a22 * KY; // d_y Q'_yyy
-    double m = (double)st.mrt[a];
-    st.Dx[a] = (fld_t<S>)(m * dQx);
-    st.Dy[a] = (fld_t<S>)(m * dQy);
 }
 
-template <class S, class A, bool FAST>
+template <class S, class A>
 __global__ void __launch_bounds__(256) k_deriv1(MeshDev M, MapStatic MS, MapScalars sc,
                                                 MapScalarsF sf, StateDev<S> st)
 {
     wait_prior_grid();
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a < M.N) deriv1_node<S, A, FAST>(M, MS, sc, sf, st, a);
+    if (a < M.N) deriv1_node<S, A>(M, MS, sc, sf, st, a);
 }
 
-template <class S, class A, bool FAST>
+// Collision of node a in the FP64 form, the fields as the moments pass left
+// them (a state that is not physical is passed on unchanged).
+__device__ __forceinline__ void collide_store64(const KinParams<double> &K, const StateDev<double> &st, int N, int a,
+                                                double Xx, double Xy)
+{
+    double f[NQ], g[NQ];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) fg_get(st.str, i, a, N, f[i], g[i]);
+    const double rho = st.rho[a], T = st.T[a];
+    if (rho > 0.0 && T > 0.0 && !(K.flags & FLAG_COLLIDE_OFF))
+        collide_node64(K, f, g, rho, st.ux[a], st.uy[a], T, st.mrt[a], Xx, Xy);
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) fg_put(st.post, i, a, N, f[i], g[i]);
+}
+
+template <class S, class A>
 __device__ __forceinline__ void collide_at(const MeshDev &M, const MapStatic &MS,
                                            const MapScalars &sc, const MapScalarsF &sf,
                                            const KinParams<A> &K, const StateDev<S> &st, int *err,
                                            int a)
 {
     const int N = M.N;
+    if constexpr (std::is_same<S, double>::value) { // from the moments pass's fields
+        double Xx = 0, Xy = 0;
+        if (!(K.flags & (FLAG_PHI_OFF | FLAG_COLLIDE_OFF))) {
+            owner_div64(M, MS, sc, st, a, st.Dx, st.Dy, Xx, Xy);
+            Xx = -Xx;
+            Xy = -Xy;
+        }
+        collide_store64(K, st, N, a, Xx, Xy);
+        return;
+    }
     A Xx = 0, Xy = 0;
-    if (FAST && !(K.flags & FLAG_PHI_OFF)) {
+    if (!(K.flags & FLAG_PHI_OFF)) {
         const FastMap F = fast_map(MS, sf, a, M.Xf[a]);
         float KX, KY;
         owner_grad_f32(M, a, st.Dx, KX, KY);
         Xx = (A)(-(F.A11 * KX + F.A21 * KY));
         owner_grad_f32(M, a, st.Dy, KX, KY);
         Xy = (A)(-(F.A12 * KX + F.A22 * KY));
-    } else if (!(K.flags & FLAG_PHI_OFF)) {
-        const double2 Xa = M.X[a];
-        double xX, xY, yX, yY, Vx, Vy, a11, a12, a21, a22;
-        map_node(MS, sc, a, Xa.x, Xa.y, xX, xY, yX, yY, Vx, Vy);
-        metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
-        double KX, KY;
-        owner_grad(M, a, st.Dx, KX, KY);
-        Xx = (A)(-(a11 * KX + a21 * KY));
-        owner_grad(M, a, st.Dy, KX, KY);
-        Xy = (A)(-(a12 * KX + a22 * KY));
     }
     A f[NQ], g[NQ];
 #pragma unroll
@@ -1264,14 +1347,14 @@ __device__ __forceinline__ void collide_at(const MeshDev &M, const MapStatic &MS
     st.T[a] = (fld_t<S>)T;
 }
 
-template <class S, class A, bool FAST>
+template <class S, class A>
 __global__ void __launch_bounds__(128) k_collide(MeshDev M, MapStatic MS, MapScalars sc,
                                                  MapScalarsF sf, KinParams<A> K, StateDev<S> st,
                                                  int *err)
 {
     wait_prior_grid();
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a < M.N) collide_at<S, A, FAST>(M, MS, sc, sf, K, st, err, a);
+    if (a < M.N) collide_at<S, A>(M, MS, sc, sf, K, st, err, a);
 }
 
 // Element choice of every population at map time t (parity report).  With

@@ -251,6 +251,10 @@ __global__ void __launch_bounds__(128) kq_fast(QuadDev M, MapStatic MS, MapScala
         if constexpr (FP64) {
             X = M.X[a];
             n = node64<TR>(MS, scd, a, X, false);
+            if (!TR && i0 == 0 && st.met) { // for the derivative passes
+                st.met[2 * a] = make_double2(n.a11, n.a12);
+                st.met[2 * a + 1] = make_double2(n.a21, n.a22);
+            }
 #pragma unroll
             for (int j = 0; j < G; ++j) c[j] = st.cache[(i0 + j) * M.N + a];
         }
@@ -308,6 +312,22 @@ __global__ void __launch_bounds__(128) kq_slow(QuadDev M, MapStatic MS, MapScala
 #endif
 static_assert(NQ % ALELB_QUAD_G == 0, "directions per thread");
 
+// d_x K0 and d_y K1 at node a in FP64 (owner_div64 on quadrilaterals).
+__device__ __forceinline__ void quad_owner_div64(const QuadDev &M, const MapStatic &MS, const MapScalars &sc,
+                                                 const StateDev<double> &st, int a, const double *K0, const double *K1,
+                                                 double &d0, double &d1)
+{
+    double X0, Y0, X1, Y1, A[4];
+    quad_owner_grad(M, a, K0, X0, Y0);
+    quad_owner_grad(M, a, K1, X1, Y1);
+    d0 = X0;
+    d1 = Y1;
+    if (MS.kind == MK_NONE || MS.kind == MK_PLUNGE) return; // A = I
+    metric64(MS, sc, M.X, st, a, A);
+    d0 = A[0] * X0 + A[2] * Y0;
+    d1 = A[1] * X1 + A[3] * Y1;
+}
+
 // D_a = (mu / rho T) d_a Q'_aaa in the owner element (Eq. Xa); FP32 in the
 // deviation forms (the FP32 map and the node's FP32 owner-element J^{-1}),
 // FP64 otherwise.
@@ -329,18 +349,11 @@ __global__ void __launch_bounds__(256) kq_deriv1(QuadDev M, MapStatic MS, MapSca
         st.Dx[a] = (fld_t<S>)(m * dQx);
         st.Dy[a] = (fld_t<S>)(m * dQy);
     } else {
-        const double2 Xa = M.X[a];
-        double xX, xY, yX, yY, Vx, Vy, a11, a12, a21, a22;
-        map_node(MS, sc, a, Xa.x, Xa.y, xX, xY, yX, yY, Vx, Vy);
-        metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
-        double KX, KY;
-        quad_owner_grad(M, a, (const double *)st.Qx, KX, KY);
-        const double dQx = a11 * KX + a21 * KY;
-        quad_owner_grad(M, a, (const double *)st.Qy, KX, KY);
-        const double dQy = a12 * KX + a22 * KY;
-        const double m = (double)st.mrt[a];
-        st.Dx[a] = (fld_t<S>)(m * dQx);
-        st.Dy[a] = (fld_t<S>)(m * dQy);
+        double dQx, dQy;
+        quad_owner_div64(M, MS, sc, st, a, st.Qx, st.Qy, dQx, dQy);
+        const double m = st.mrt[a];
+        st.Dx[a] = m * dQx;
+        st.Dy[a] = m * dQy;
     }
 }
 
@@ -353,8 +366,17 @@ __global__ void __launch_bounds__(128) kq_collide(QuadDev M, MapStatic MS, MapSc
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= M.N) return;
     const int N = M.N;
-    A Xx = 0, Xy = 0;
-    if constexpr (!std::is_same<S, double>::value) {
+    if constexpr (std::is_same<S, double>::value) { // from the moments pass's fields
+        double Xx = 0, Xy = 0;
+        if (!(K.flags & (FLAG_PHI_OFF | FLAG_COLLIDE_OFF))) {
+            quad_owner_div64(M, MS, sc, st, a, st.Dx, st.Dy, Xx, Xy);
+            Xx = -Xx;
+            Xy = -Xy;
+        }
+        collide_store64(K, st, N, a, Xx, Xy);
+        return;
+    } else {
+        A Xx = 0, Xy = 0;
         if (!(K.flags & FLAG_PHI_OFF)) {
             const FastMap F = fast_map(MS, sf, a, M.Xf[a]);
             float KX, KY;
@@ -363,28 +385,18 @@ __global__ void __launch_bounds__(128) kq_collide(QuadDev M, MapStatic MS, MapSc
             quad_owner_grad(M, a, st.Dy, KX, KY);
             Xy = (A)(-(F.A12 * KX + F.A22 * KY));
         }
-    } else if (!(K.flags & FLAG_PHI_OFF)) {
-        const double2 Xa = M.X[a];
-        double xX, xY, yX, yY, Vx, Vy, a11, a12, a21, a22;
-        map_node(MS, sc, a, Xa.x, Xa.y, xX, xY, yX, yY, Vx, Vy);
-        metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
-        double KX, KY;
-        quad_owner_grad(M, a, (const double *)st.Dx, KX, KY);
-        Xx = (A)(-(a11 * KX + a21 * KY));
-        quad_owner_grad(M, a, (const double *)st.Dy, KX, KY);
-        Xy = (A)(-(a12 * KX + a22 * KY));
+        A f[NQ], g[NQ];
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) fg_get(st.str, i, a, N, f[i], g[i]);
+        A rho, ux, uy, T;
+        if (!collide_node(K, f, g, Xx, Xy, rho, ux, uy, T)) atomicOr(err, ERR_NONFINITE);
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) fg_put(st.post, i, a, N, f[i], g[i]);
+        st.rho[a] = (fld_t<S>)rho;
+        st.ux[a] = (fld_t<S>)ux;
+        st.uy[a] = (fld_t<S>)uy;
+        st.T[a] = (fld_t<S>)T;
     }
-    A f[NQ], g[NQ];
-#pragma unroll
-    for (int i = 0; i < NQ; ++i) fg_get(st.str, i, a, N, f[i], g[i]);
-    A rho, ux, uy, T;
-    if (!collide_node(K, f, g, Xx, Xy, rho, ux, uy, T)) atomicOr(err, ERR_NONFINITE);
-#pragma unroll
-    for (int i = 0; i < NQ; ++i) fg_put(st.post, i, a, N, f[i], g[i]);
-    st.rho[a] = (fld_t<S>)rho;
-    st.ux[a] = (fld_t<S>)ux;
-    st.uy[a] = (fld_t<S>)uy;
-    st.T[a] = (fld_t<S>)T;
 }
 
 // Element choice of every population (parity report): original element id,

@@ -374,6 +374,18 @@ ALELB_HD __forceinline__ bool quad_local(const QuadDev &M, int e, int sx, int sy
     return quad_newton_t<A>(c, A(1e-5), A(1e-4), xi, eta); // FP32: converged near 1e-7
 }
 
+// FP64 <-> FP32 by their bits, for values whose rounding does not matter
+// (the FP64 pipe runs conversions at its own low rate): truncation toward
+// zero, below the normal range to zero, above it to the largest float.
+__device__ __forceinline__ float d2f_bits(double v)
+{
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v), m = hi & 0x7fffffffu;
+    unsigned b = ((m - 0x38000000u) << 3) | (lo >> 29);
+    if (m < 0x38100000u) b = 0u;
+    if (m >= 0x47f00000u) b = 0x7f7fffffu;
+    return __uint_as_float(b | (hi & 0x80000000u));
+}
+
 // Local coordinates of p in element e for the FP64 form: Newton in FP32 on
 // the bilinear map x = b0 + b1 xi + b2 eta + b3 xi eta, then two corrections
 // with the residual in FP64 and the FP32 inverse Jacobian.  A correction
@@ -390,9 +402,9 @@ __device__ __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, in
     if (sx) b0.x = da(b0.x, sx * M.Lx);
     if (sy) b0.y = da(b0.y, sy * M.Ly);
     const double dx = ds(px, b0.x), dy = ds(py, b0.y);
-    const float fx = (float)dx, fy = (float)dy;
-    const float b1x = (float)b1.x, b1y = (float)b1.y, b2x = (float)b2.x, b2y = (float)b2.y, b3x = (float)b3.x,
-                b3y = (float)b3.y;
+    const float fx = d2f_bits(dx), fy = d2f_bits(dy);
+    const float b1x = d2f_bits(b1.x), b1y = d2f_bits(b1.y), b2x = d2f_bits(b2.x), b2y = d2f_bits(b2.y),
+                b3x = d2f_bits(b3.x), b3y = d2f_bits(b3.y);
     float u = 0.f, v = 0.f, i11 = 0.f, i12 = 0.f, i21 = 0.f, i22 = 0.f;
     const auto inverse = [&]() { // J^{-1} at (u, v)
         const float j11 = __fmaf_rn(b3x, v, b1x), j12 = __fmaf_rn(b3x, u, b2x);
@@ -415,18 +427,18 @@ __device__ __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, in
         if (fabsf(du) + fabsf(dv) < 1e-4f) break; // the next step would be below the FP32 rounding
     }
     inverse();
-    xi = (double)u;
-    eta = (double)v;
+    xi = f2d_bits(u);
+    eta = f2d_bits(v);
     float du = 0.f, dv = 0.f;
 #pragma unroll
     for (int it = 0; it < 2; ++it) {
         const double q = dm(xi, eta);
-        const float rx = (float)ds(dx, dfma(b3.x, q, dfma(b2.x, eta, dm(b1.x, xi))));
-        const float ry = (float)ds(dy, dfma(b3.y, q, dfma(b2.y, eta, dm(b1.y, xi))));
+        const float rx = d2f_bits(ds(dx, dfma(b3.x, q, dfma(b2.x, eta, dm(b1.x, xi)))));
+        const float ry = d2f_bits(ds(dy, dfma(b3.y, q, dfma(b2.y, eta, dm(b1.y, xi)))));
         du = __fmaf_rn(i11, rx, __fmul_rn(i12, ry));
         dv = __fmaf_rn(i21, rx, __fmul_rn(i22, ry));
-        xi = da(xi, (double)du);
-        eta = da(eta, (double)dv);
+        xi = da(xi, f2d_bits(du));
+        eta = da(eta, f2d_bits(dv));
     }
     return fabsf(du) <= 1e-9f && fabsf(dv) <= 1e-9f;
 }

@@ -150,6 +150,11 @@ inline MapScalars map_scalars(int kind, const double *p, double t)
             S.vy = -(h * omh) * std::cos(omh * t);
         }
     }
+    if (kind == MK_PITCH || kind == MK_PITCH_PLUNGE) {
+        metric_inverse_T(S.c, -S.sn, S.sn, S.c, S.A11, S.A12, S.A21, S.A22);
+    } else if (uniform_metric(kind)) {
+        S.A11 = S.A22 = 1.0;
+    }
     return S;
 }
 
