@@ -1152,7 +1152,8 @@ ALELB_HD __forceinline__ bool fast_decide(const MeshDev &M, const FastMap &F, fl
 // node then lie outside the closed mesh.  Returns the boundary kind, or 0
 // when not certain.  Errors: F.eq(i) per component of -c^, the FP32
 // rounding of the edge vectors and of the cross products.
-ALELB_HD __forceinline__ int cone_missing(const MeshDev &M, const FastMap &F, int a, int i)
+template <class Mesh> // MeshDev or QuadDev
+ALELB_HD __forceinline__ int cone_missing(const Mesh &M, const FastMap &F, int a, int i)
 {
     const int ck = M.conek[a];
     if (!ck) return 0;

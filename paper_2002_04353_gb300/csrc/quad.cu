@@ -25,15 +25,18 @@ namespace {
 // FP32, the nine-node interpolation.  False: left to the exact path.
 template <class S, class A>
 __device__ __forceinline__ bool quad_fast_pop(const QuadDev &M, const FastMap &F, float4 Xf, const StateDev<S> &st,
-                                              int a, int i)
+                                              int a, int i, unsigned lanes)
 {
     const int N = M.N;
     const int c = st.cache[i * N + a];
-    int e;
+    int e = 0;
     float cw[8];
     float xi, eta;
-    if (!(quad_fast_decide(M, F, Xf, a, i, c, e, cw) && quad_newton_t<float>(cw, 1e-5f, 1e-4f, xi, eta)))
-        return false;
+    bool in = quad_fast_decide(M, F, Xf, a, i, c, e, cw);
+    __syncwarp(lanes);
+    if (in) in = quad_newton_t<float>(cw, 1e-5f, 1e-4f, xi, eta);
+    __syncwarp(lanes);
+    if (!in) return false;
     A Nw[9];
     shape9<A>((A)xi, (A)eta, Nw);
     A fi = 0, gi = 0;
@@ -53,17 +56,98 @@ __device__ __forceinline__ bool quad_fast_pop(const QuadDev &M, const FastMap &F
 // point, local coordinates and interpolation in FP64.
 template <bool TR>
 __device__ __forceinline__ bool quad_fast_pop64(const QuadDev &M, const FastMap &F, const Node64 &n, float4 Xf, double2 X,
-                                                const StateDev<double> &st, int a, int i, int c)
+                                                const StateDev<double> &st, int a, int i, int c, unsigned lanes)
 {
-    int e;
+    int e = 0;
     float cw[8];
-    if (!quad_fast_decide(M, F, Xf, a, i, c, e, cw)) return false;
     double px, py, xi, eta, f, g;
-    departure64<TR>(n, i, X, px, py);
-    if (!quad_local64(M, e, 0, 0, px, py, xi, eta)) return false;
+    bool in = quad_fast_decide(M, F, Xf, a, i, c, e, cw);
+    __syncwarp(lanes);
+    if (in) {
+        departure64<TR>(n, i, X, px, py);
+        in = quad_local64(M, e, 0, 0, px, py, xi, eta);
+    }
+    __syncwarp(lanes);
+    if (!in) return false;
     quad_interp64(M, st.post, M.N, i, e, xi, eta, f, g);
     fg_put(st.str, i, a, M.N, f, g);
     return true;
+}
+
+// Missing populations of Sec. IV.A at node a (all nine directions), from its
+// metrics and mesh velocity at the arrival time.
+template <class S, class A>
+__device__ __forceinline__ void quad_missing(const QuadDev &M, const KinParams<A> &K, const StateDev<S> &st, int a,
+                                             double a11, double a12, double a21, double a22, double Vx, double Vy,
+                                             A fm[NQ], A gm[NQ])
+{
+    A rt, uxt, uyt, Tt;
+    const int wi = M.wall_idx[a];
+    if (wi >= 0) { // wall node: u = V_G, rho and T at the probe B
+        const int pe = M.probe_e[wi];
+        const double2 pxi = M.probe_xi[wi];
+        A Nw[9];
+        shape9<A>((A)pxi.x, (A)pxi.y, Nw);
+        A r = 0, t = 0, ub = 0, vb = 0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int b = M.conn[9 * pe + k];
+            r += Nw[k] * (A)st.rho[b];
+            t += Nw[k] * (A)st.T[b];
+            if (K.flags & FLAG_SLIP) {
+                ub += Nw[k] * (A)st.ux[b];
+                vb += Nw[k] * (A)st.uy[b];
+            }
+        }
+        rt = r;
+        Tt = t;
+        uxt = (A)Vx;
+        uyt = (A)Vy;
+        if (K.flags & FLAG_SLIP) {
+            const double2 nw = M.wall_nrm[wi];
+            slip_target<A>((A)a11, (A)a12, (A)a21, (A)a22, (A)nw.x, (A)nw.y, ub, vb, (A)Vx, (A)Vy, uxt, uyt);
+        }
+    } else { // off-wall node: its previous-step fields (mesh velocity under R8c)
+        const bool vg = (K.flags & FLAG_OFFWALL_VG) != 0;
+        rt = (A)st.rho[a];
+        uxt = vg ? (A)Vx : (A)st.ux[a];
+        uyt = vg ? (A)Vy : (A)st.uy[a];
+        Tt = (A)st.T[a];
+    }
+    A du[4] = {0, 0, 0, 0}, dT[2] = {0, 0};
+    if (!(K.flags & FLAG_BC_EQ) && !((K.flags & FLAG_SLIP) && wi >= 0)) {
+        double G[6];
+        quad_grad3_linear(M, M.bcel[a], st.ux, st.uy, st.T, G);
+        du[0] = (A)(a11 * G[0] + a21 * G[1]);
+        du[1] = (A)(a12 * G[0] + a22 * G[1]);
+        du[2] = (A)(a11 * G[2] + a21 * G[3]);
+        du[3] = (A)(a12 * G[2] + a22 * G[3]);
+        dT[0] = (A)(a11 * G[4] + a21 * G[5]);
+        dT[1] = (A)(a12 * G[4] + a22 * G[5]);
+    }
+    grad_missing(K, rt, uxt, uyt, Tt, du, dT, fm, gm);
+}
+// The same with the map evaluated, the directions in mask written.
+template <class S, class A>
+__device__ __forceinline__ void quad_bc_node(const QuadDev &M, const MapStatic &MS, const MapScalars &sc,
+                                             const KinParams<A> &K, const StateDev<S> &st, int a, unsigned mask)
+{
+    const double2 X = M.X[a];
+    double xX, xY, yX, yY, Vx, Vy, a11, a12, a21, a22;
+    map_node(MS, sc, a, X.x, X.y, xX, xY, yX, yY, Vx, Vy);
+    if (uniform_metric(MS.kind)) {
+        a11 = sc.A11;
+        a12 = sc.A12;
+        a21 = sc.A21;
+        a22 = sc.A22;
+    } else {
+        metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
+    }
+    A fm[NQ], gm[NQ];
+    quad_missing(M, K, st, a, a11, a12, a21, a22, Vx, Vy, fm, gm);
+#pragma unroll
+    for (int i = 0; i < NQ; ++i)
+        if (mask >> i & 1u) fg_put(st.str, i, a, M.N, fm[i], gm[i]);
 }
 
 // Propagation of population pairs i0 .. i0 + G - 1 of node a on the exact
@@ -150,54 +234,7 @@ __device__ __forceinline__ unsigned quad_stream_pops(const QuadDev &M, const Map
         }
         A fm[NQ], gm[NQ];
         if (miss & ~far) {
-            A rt, uxt, uyt, Tt;
-            const int wi = M.wall_idx[a];
-            if (wi >= 0) { // wall node: u = V_G, rho and T at the probe B
-                const int pe = M.probe_e[wi];
-                const double2 pxi = M.probe_xi[wi];
-                A Nw[9];
-                shape9<A>((A)pxi.x, (A)pxi.y, Nw);
-                A r = 0, t = 0, ub = 0, vb = 0;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const int b = M.conn[9 * pe + k];
-                    r += Nw[k] * (A)st.rho[b];
-                    t += Nw[k] * (A)st.T[b];
-                    if (K.flags & FLAG_SLIP) {
-                        ub += Nw[k] * (A)st.ux[b];
-                        vb += Nw[k] * (A)st.uy[b];
-                    }
-                }
-                rt = r;
-                Tt = t;
-                uxt = (A)Vx;
-                uyt = (A)Vy;
-                if (K.flags & FLAG_SLIP) {
-                    const double2 nw = M.wall_nrm[wi];
-                    slip_target<A>((A)a11, (A)a12, (A)a21, (A)a22, (A)nw.x, (A)nw.y, ub, vb, (A)Vx, (A)Vy, uxt, uyt);
-                }
-            } else { // off-wall node: its previous-step fields (mesh velocity under R8c)
-                const bool vg = (K.flags & FLAG_OFFWALL_VG) != 0;
-                rt = (A)st.rho[a];
-                uxt = vg ? (A)Vx : (A)st.ux[a];
-                uyt = vg ? (A)Vy : (A)st.uy[a];
-                Tt = (A)st.T[a];
-            }
-            A du[4] = {0, 0, 0, 0}, dT[2] = {0, 0};
-            if (!(K.flags & FLAG_BC_EQ) && !((K.flags & FLAG_SLIP) && wi >= 0)) {
-                const int2 bc = M.bcel[a];
-                double KX, KY;
-                quad_grad(M, bc, st.ux, false, KX, KY);
-                du[0] = (A)(a11 * KX + a21 * KY);
-                du[1] = (A)(a12 * KX + a22 * KY);
-                quad_grad(M, bc, st.uy, false, KX, KY);
-                du[2] = (A)(a11 * KX + a21 * KY);
-                du[3] = (A)(a12 * KX + a22 * KY);
-                quad_grad(M, bc, st.T, false, KX, KY);
-                dT[0] = (A)(a11 * KX + a21 * KY);
-                dT[1] = (A)(a12 * KX + a22 * KY);
-            }
-            grad_missing(K, rt, uxt, uyt, Tt, du, dT, fm, gm);
+            quad_missing(M, K, st, a, a11, a12, a21, a22, Vx, Vy, fm, gm);
         }
 #pragma unroll
         for (int i = 0; i < NQ; ++i) {
@@ -208,6 +245,67 @@ __device__ __forceinline__ unsigned quad_stream_pops(const QuadDev &M, const Map
         }
     }
     return walks;
+}
+
+// Population i of node a on the exact path, its walk on certified FP32
+// predicates: location, interpolation, far-field or wall condition.  Returns
+// the number of walks (0: c^ is exactly zero).  Where no FP32 map is usable the
+// FP64 departure point is walked (quad_stream_pops).
+template <class S, class A>
+__device__ __forceinline__ unsigned quad_slow_pop(const QuadDev &M, const MapStatic &MS, const MapScalars &sc,
+                                                  const MapScalars &scd, const MapScalarsF &sfd, const KinParams<A> &K,
+                                                  const StateDev<S> &st, int *err, int a, int i)
+{
+    const int N = M.N;
+    prefetch_l1(M.X + a);
+    prefetch_l1(M.fan_ptr + a);
+    prefetch_l1(M.wall_idx + a);
+    const float4 Xf = M.Xf[a];
+    const FastMap F = fast_map(MS, sfd, a, Xf);
+    const float cx = (float)lat_cx(i), cy = (float)lat_cy(i);
+    const float chx = F.A11 * cx + F.A12 * cy - F.W1;
+    const float chy = F.A21 * cx + F.A22 * cy - F.W2;
+    if ((K.flags & (FLAG_LITERAL_VG | FLAG_EXACT_CHAR)) || !F.ok || !(sqrtf(chx * chx + chy * chy) > 4.0f * F.eq(i)))
+        return quad_stream_pops<1, true>(M, MS, sc, scd, K, st, err, a, i);
+    QPred32 pr{M, MS, scd, a, i, Xf, -chx, -chy, F.eq(i)};
+    pr.have64 = false;
+    const Loc L = quad_walk_t(M, pr, a, err);
+    st.cache[i * N + a] = L.e >= 0 ? (L.e | ((L.sx + 1) << 28) | ((L.sy + 1) << 30)) : -1;
+    if (L.e == -1) {
+        if (L.kind == 2) fg_put(st.str, i, a, N, K.finf[i], K.ginf[i]);
+        else quad_bc_node(M, MS, sc, K, st, a, 1u << i);
+        return 1u;
+    }
+    A fi = 0, gi = 0;
+    if (L.e == -2 || L.vnode >= 0) {
+        fg_get(st.post, i, L.e == -2 ? a : L.vnode, N, fi, gi);
+    } else if constexpr (std::is_same<S, double>::value) {
+        const double2 X = M.X[a];
+        const Node64 n = node64<false>(MS, scd, a, X, false);
+        double px, py, xi, eta;
+        departure64<false>(n, i, X, px, py);
+        if (!quad_local64(M, L.e, L.sx, L.sy, px, py, xi, eta) &&
+            !quad_local<double>(M, L.e, L.sx, L.sy, px, py, xi, eta))
+            set_err(err, ERR_LOCATE);
+        quad_interp64(M, st.post, N, i, L.e, xi, eta, fi, gi);
+    } else {
+        pr.load(L.e, L.sx, L.sy); // the walk may end in the neighbour across an edge
+        const float c[8] = {pr.x0 + chx, pr.y0 + chy, pr.x1 + chx, pr.y1 + chy,
+                            pr.x2 + chx, pr.y2 + chy, pr.x3 + chx, pr.y3 + chy};
+        float xi, eta;
+        if (!quad_newton_t<float>(c, 1e-5f, 1e-4f, xi, eta)) set_err(err, ERR_LOCATE);
+        A Nw[9];
+        shape9<A>((A)xi, (A)eta, Nw);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            A fb, gb;
+            fg_get(st.post, i, M.conn[9 * L.e + k], N, fb, gb);
+            fi += Nw[k] * fb;
+            gi += Nw[k] * gb;
+        }
+    }
+    fg_put(st.str, i, a, N, fi, gi);
+    return 1u;
 }
 
 // Grid (node blocks, 9 / G direction groups): G directions per thread.
@@ -230,10 +328,14 @@ __global__ void __launch_bounds__(128) kq_stream(QuadDev M, MapStatic MS, MapSca
 // (grid y: 9 / G direction groups, G directions per thread) and lists the
 // others; kq_slow runs the exact path over the list, spread over all blocks,
 // so that the walks do not hold up the warps of settled populations.  TR: the
-// map is a translation (no map, plunge).
+// map is a translation (no map, plunge).  The lanes are brought together after
+// the certified test and after Newton (__syncwarp): left apart, the own and the
+// other elements' lanes interpolated one after the other (150,400 nodes: 60 us
+// against 33 in FP32, 408 against 175 in FP64).  FP32 is held to 32 registers,
+// 16 blocks an SM (35 us at 40).
 template <class S, class A, int G, bool TR>
-__global__ void __launch_bounds__(128) kq_fast(QuadDev M, MapStatic MS, MapScalars scd, MapScalarsF sfd,
-                                               KinParams<A> K, StateDev<S> st)
+__global__ void __launch_bounds__(128, std::is_same<S, double>::value ? 1 : 16) kq_fast(QuadDev M, MapStatic MS, MapScalars scd, MapScalarsF sfd,
+                                               KinParams<A> K, StateDev<S> st, unsigned long long *stats)
 {
     constexpr bool FP64 = std::is_same<S, double>::value;
     wait_prior_grid();
@@ -241,6 +343,7 @@ __global__ void __launch_bounds__(128) kq_fast(QuadDev M, MapStatic MS, MapScala
     int code[G];
 #pragma unroll
     for (int j = 0; j < G; ++j) code[j] = 0;
+    const unsigned lanes = __ballot_sync(0xffffffffu, a < M.N);
     if (a < M.N) {
         const float4 Xf = M.Xf[a];
         FastMap F = TR ? fast_map_translation(sfd, Xf) : fast_map(MS, sfd, a, Xf);
@@ -261,12 +364,22 @@ __global__ void __launch_bounds__(128) kq_fast(QuadDev M, MapStatic MS, MapScala
 #pragma unroll
         for (int j = 0; j < G; ++j) {
             const int i = i0 + j;
+            __syncwarp(lanes);
+            // (a node of zero mesh velocity fails the test: its c^_0 is zero)
+            bool done;
+            if constexpr (FP64) done = quad_fast_pop64<TR>(M, F, n, Xf, X, st, a, i, c[j], lanes);
+            else done = quad_fast_pop<S, A>(M, F, Xf, st, a, i, lanes);
+            if (!done && F.ok) {
+                const int ck = cone_missing(M, F, a, i);
+                if (ck == 2) fg_put(st.str, i, a, M.N, K.finf[i], K.ginf[i]); // far field
+                // 3: settled, but not by the element (the counter tells them apart)
+                code[j] = ck == 2 ? 3 : ck == 1 ? 2 : 1;
+            } else {
+                code[j] = done ? 0 : 1;
+            }
             if (i == 0 && M.vzero[a] && !(K.flags & FLAG_SHIFT)) { // c^_0 exactly zero: the node's own value
                 fg_copy(st.str, st.post, 0, a, M.N);
-            } else if constexpr (FP64) {
-                code[j] = F.ok && quad_fast_pop64<TR>(M, F, n, Xf, X, st, a, i, c[j]) ? 0 : 1;
-            } else {
-                code[j] = F.ok && quad_fast_pop<S, A>(M, F, Xf, st, a, i) ? 0 : 1;
+                code[j] = 0;
             }
         }
     }
@@ -275,16 +388,25 @@ __global__ void __launch_bounds__(128) kq_fast(QuadDev M, MapStatic MS, MapScala
     for (int j = 0; j < G; ++j) any |= code[j];
     if (__any_sync(0xffffffffu, any != 0)) {
 #pragma unroll
-        for (int j = 0; j < G; ++j) append_pop(st, a, M.N, i0 + j, code[j]);
+        for (int j = 0; j < G; ++j) {
+            append_pop(st, a, M.N, i0 + j, code[j]);
+            const unsigned far = __ballot_sync(0xffffffffu, code[j] == 3);
+            if (!FP64 && stats && far && (threadIdx.x & 31u) == 0u) atomicAdd(stats, (unsigned long long)__popc(far));
+        }
     }
 }
 
+// The exact path's walk runs on certified FP32 signs, the wall condition once
+// per wall node for its cone-certified directions, its three gradients with one
+// Jacobian: 31 us against 53 with every listed population walked in FP64 and
+// its wall condition computed per direction (FP32, 150,400 nodes; FP64 form 43
+// against 67).  Bound by the latency of one entry's chain.
 // The counter: the deviation forms count the populations that the certified
 // test does not settle (the nodes of zero mesh velocity among them), the FP64
 // form all that are located (9 N less those whose c^ is exactly zero).
 template <class S, class A>
-__global__ void __launch_bounds__(128) kq_slow(QuadDev M, MapStatic MS, MapScalars sc, MapScalars scd, KinParams<A> K,
-                                               StateDev<S> st, int *err, unsigned long long *stats)
+__global__ void __launch_bounds__(128) kq_slow(QuadDev M, MapStatic MS, MapScalars sc, MapScalars scd, MapScalarsF sfd,
+                                               KinParams<A> K, StateDev<S> st, int *err, unsigned long long *stats)
 {
     constexpr bool FP64 = std::is_same<S, double>::value;
     wait_prior_grid();
@@ -296,10 +418,18 @@ __global__ void __launch_bounds__(128) kq_slow(QuadDev M, MapStatic MS, MapScala
         const unsigned nz = K.flags & FLAG_SHIFT ? 0u : (unsigned)M.nvzero;
         atomicAdd(stats, FP64 ? (unsigned long long)NQ * M.N - nz : (unsigned long long)n + nz);
     }
-    for (unsigned w = spread_first(); w < n; w += spread_stride()) {
-        const int code = work_at(st.work, M.N, pre, w);
-        const unsigned walks = quad_stream_pops<1, true>(M, MS, sc, scd, K, st, err, code / NQ, code % NQ);
-        if (FP64 && stats && !walks) atomicAdd(stats, ~0ull); // c^ exactly zero: one less
+    const unsigned total = n + st.wcount[NQ]; // then the wall nodes, with their certified directions
+    for (unsigned w = spread_first(); w < total; w += spread_stride()) {
+        if (w < n) {
+            const int code = work_at(st.work, M.N, pre, w);
+            const unsigned walks = quad_slow_pop(M, MS, sc, scd, sfd, K, st, err, code / NQ, code % NQ);
+            if (FP64 && stats && !walks) atomicAdd(stats, ~0ull); // c^ exactly zero: one less
+        } else {
+            const int a = st.work[(size_t)NQ * M.N + (w - n)];
+            const unsigned mask = st.wmask[a] & WMASK_DIRS;
+            if (!FP64 && stats) atomicAdd(stats, (unsigned long long)__popc(mask));
+            quad_bc_node(M, MS, sc, K, st, a, mask);
+        }
     }
 }
 
@@ -456,10 +586,10 @@ __global__ void __launch_bounds__(256) kq_forces(QuadDev M, MapStatic MS, MapSca
             map_node(MS, sc, a, Xa.x, Xa.y, xX, xY, yX, yY, Vx, Vy);
             metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
             double KX, KY, d[4];
-            quad_grad(M, M.owner[a], st.ux, true, KX, KY);
+            quad_grad(M, M.owner[a], st.ux, KX, KY);
             d[0] = a11 * KX + a21 * KY;
             d[1] = a12 * KX + a22 * KY;
-            quad_grad(M, M.owner[a], st.uy, true, KX, KY);
+            quad_grad(M, M.owner[a], st.uy, KX, KY);
             d[2] = a11 * KX + a21 * KY;
             d[3] = a12 * KX + a22 * KY;
             const double div = d[0] + d[3];
@@ -518,6 +648,8 @@ alelb_status quad_mesh_upload(alelb_mesh *m)
     D.ownJf = B.put(Q.ownJf, st);
     D.ownJd = B.put(Q.ownJd, st);
     D.ebd = B.put(Q.ebd, st);
+    D.cone = B.put(Q.cone, st);
+    D.conek = B.put(Q.conek, st);
     D.vzero = B.put(Q.vzero, st);
     D.nvzero = (int)std::count(Q.vzero.begin(), Q.vzero.end(), (uint8_t)1);
     m->d_wedges = B.put(Q.wedges, st);
@@ -554,7 +686,7 @@ cudaError_t quad_launch(alelb_solver *s, int kernel, const MapScalars &sc, const
             const bool tr = m->T.mkind == MK_NONE || m->T.mkind == MK_PLUNGE;
             const dim3 gb(128), g1((N + 127) / 128, NQ), g3(g1.x, NQ / 3);
             if (tr) {
-                launch_pdl(kq_fast<S, A, 1, true>, g1, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st);
+                launch_pdl(kq_fast<S, A, 1, true>, g1, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st, s->d_stats);
                 break;
             }
             if constexpr (std::is_same<S, double>::value) {
@@ -563,11 +695,11 @@ cudaError_t quad_launch(alelb_solver *s, int kernel, const MapScalars &sc, const
                 // per thread; 160k box 280, 318, 326; 24k 54, 62, 80), one per
                 // direction below (1k box: 13, 24, 58 us)
                 if (N >= FAST64_G3_NODES) {
-                    launch_pdl(kq_fast<S, A, 3, false>, g3, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st);
+                    launch_pdl(kq_fast<S, A, 3, false>, g3, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st, s->d_stats);
                     break;
                 }
             }
-            launch_pdl(kq_fast<S, A, 1, false>, g1, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st);
+            launch_pdl(kq_fast<S, A, 1, false>, g1, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st, s->d_stats);
             break;
         }
         case KT_SLOW: {
@@ -577,8 +709,8 @@ cudaError_t quad_launch(alelb_solver *s, int kernel, const MapScalars &sc, const
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kq_slow<S, A>, 128, 0);
                 return v > 0 ? v : 1;
             }();
-            launch_pdl(kq_slow<S, A>, dim3(per_sm * s->n_sm), dim3(128), s->stream, m->qdev, m->mst, sc, scd, K, st,
-                       s->d_err, s->d_stats);
+            launch_pdl(kq_slow<S, A>, dim3(per_sm * s->n_sm), dim3(128), s->stream, m->qdev, m->mst, sc, scd,
+                       to_f32(scd, m->T), K, st, s->d_err, s->d_stats);
             break;
         }
         case KT_MOMENTS:

@@ -35,6 +35,8 @@ struct QuadTables {
     std::vector<double2> ownJd; // [2N]
     std::vector<double2> ebd;   // [4E] b0, b1, b2, b3: x = b0 + b1 xi + b2 eta + b3 xi eta
     std::vector<uint8_t> vzero; // [N]
+    std::vector<float4> cone;   // [N] exterior cones (build_cones)
+    std::vector<uint8_t> conek; // [N]
 };
 
 // Local coordinates of p in the quadrilateral with corners w (x, y pairs),
@@ -255,6 +257,18 @@ inline alelb_status build_quad_tables(const alelb_mesh_desc *d, HostTables &T, Q
                 }
             }
         }
+    {
+        std::vector<BoundaryEdge> be;
+        for (int en = 0; en < E; ++en)
+            for (int k = 0; k < 4; ++k) {
+                const int kind = (int)((Q.einfo[en] >> (8 * k)) & 3u);
+                if (!kind) continue;
+                const int k1 = (k + 1) % 4;
+                be.push_back({Q.conn[9 * en + k], Q.conn[9 * en + k1], Q.conn[9 * en + 4 + k],
+                              Q.ev[4 * en + k1].x - Q.ev[4 * en + k].x, Q.ev[4 * en + k1].y - Q.ev[4 * en + k].y, kind});
+            }
+        build_cones(N, be, Q.cone, Q.conek);
+    }
     // wall-condition gradient element (reading R8): among the incident
     // elements with a corner on a wall edge the one of larger area, then
     // lower original id; the owner when none touches a wall.  (elem, local)

@@ -158,6 +158,45 @@ inline MapScalars map_scalars(int kind, const double *p, double t)
     return S;
 }
 
+// Exterior cone of each boundary node: its outgoing and incoming boundary
+// edges (the domain on their left) when it has exactly one of each, of one
+// kind; a departure direction strictly right of both leaves the mesh at once
+// (the population is missing).  conek: the kind; | 4 at a convex corner of
+// the domain (the boundary turns left by a clear margin), where the domain
+// near the node is the intersection of the two left half-planes, so leaving
+// across either edge line leaves the mesh; | 8 at a reflex corner (turns right
+// by a clear margin), where the domain near the node is their union.
+struct BoundaryEdge {
+    int va, vb, mid; // from va to vb, the midside node
+    double ex, ey;   // vb - va
+    int kind;
+};
+inline void build_cones(int N, const std::vector<BoundaryEdge> &be, std::vector<float4> &cone, std::vector<uint8_t> &conek)
+{
+    std::vector<int> nout(N, 0), nin(N, 0), kk(N, 0);
+    cone.assign(N, make_float4(0, 0, 0, 0));
+    conek.assign(N, 0);
+    for (const BoundaryEdge &b : be) {
+        auto add = [&](int node, bool out, double x, double y) {
+            if (kk[node] && kk[node] != b.kind) kk[node] = -1;
+            else if (!kk[node]) kk[node] = b.kind;
+            if (out) { nout[node]++; cone[node].x = (float)x; cone[node].y = (float)y; }
+            else { nin[node]++; cone[node].z = (float)x; cone[node].w = (float)y; }
+        };
+        add(b.va, true, b.ex, b.ey);
+        add(b.vb, false, b.ex, b.ey);
+        add(b.mid, true, 0.5 * b.ex, 0.5 * b.ey);
+        add(b.mid, false, 0.5 * b.ex, 0.5 * b.ey);
+    }
+    for (int a = 0; a < N; ++a)
+        if (nout[a] == 1 && nin[a] == 1 && kk[a] > 0) {
+            const double ox = cone[a].x, oy = cone[a].y, ix = cone[a].z, iy = cone[a].w;
+            const double cr = ix * oy - iy * ox;
+            const double tol = 1e-6 * std::sqrt((ix * ix + iy * iy) * (ox * ox + oy * oy));
+            conek[a] = (uint8_t)(kk[a] | (cr > tol ? 4 : 0) | (cr < -tol ? 8 : 0));
+        }
+}
+
 // Validates the description and fills T.  Returns ALELB_OK or an error
 // with a message in err.
 // Neighbour ring of each node for the learned departure-element proposal:
@@ -493,44 +532,18 @@ inline alelb_status build_tables(const alelb_mesh_desc *d, HostTables &T, std::s
                 }
             }
         }
-    // exterior cone of each boundary node: its outgoing and incoming boundary
-    // edges (the domain on their left) when it has exactly one of each, of
-    // one kind; a departure direction strictly right of both leaves the mesh
-    // at once (the population is missing)
+    // exterior cones (build_cones) from the boundary edges in element order
     {
-        std::vector<int> nout(N, 0), nin(N, 0), kk(N, 0);
-        T.cone.assign(N, make_float4(0, 0, 0, 0));
-        T.conek.assign(N, 0);
+        std::vector<BoundaryEdge> be;
         for (int en = 0; en < E; ++en)
             for (int k = 0; k < 3; ++k) {
                 const int kind = (int)((einfo[en] >> (8 * k)) & 3u);
                 if (!kind) continue;
                 const int k1 = (k + 1) % 3;
-                const double ex = ev[3 * en + k1].x - ev[3 * en + k].x, ey = ev[3 * en + k1].y - ev[3 * en + k].y;
-                const int va = conn[6 * en + k], vb = conn[6 * en + k1], mid = conn[6 * en + 3 + k];
-                auto add = [&](int node, bool out, double x, double y) {
-                    if (kk[node] && kk[node] != kind) kk[node] = -1;
-                    else if (!kk[node]) kk[node] = kind;
-                    if (out) { nout[node]++; T.cone[node].x = (float)x; T.cone[node].y = (float)y; }
-                    else { nin[node]++; T.cone[node].z = (float)x; T.cone[node].w = (float)y; }
-                };
-                add(va, true, ex, ey);
-                add(vb, false, ex, ey);
-                add(mid, true, 0.5 * ex, 0.5 * ey);
-                add(mid, false, 0.5 * ex, 0.5 * ey);
+                be.push_back({conn[6 * en + k], conn[6 * en + k1], conn[6 * en + 3 + k],
+                              ev[3 * en + k1].x - ev[3 * en + k].x, ev[3 * en + k1].y - ev[3 * en + k].y, kind});
             }
-        // bit 2: a convex corner of the domain (the boundary turns left by a
-        // clear margin), where the domain near the node is the intersection
-        // of the two left half-planes, so leaving across either edge line
-        // leaves the mesh; bit 3: a reflex corner (turns right by a clear
-        // margin), where the domain near the node is their union
-        for (int a = 0; a < N; ++a)
-            if (nout[a] == 1 && nin[a] == 1 && kk[a] > 0) {
-                const double ox = T.cone[a].x, oy = T.cone[a].y, ix = T.cone[a].z, iy = T.cone[a].w;
-                const double cr = ix * oy - iy * ox;
-                const double tol = 1e-6 * std::sqrt((ix * ix + iy * iy) * (ox * ox + oy * oy));
-                T.conek[a] = (uint8_t)(kk[a] | (cr > tol ? 4 : 0) | (cr < -tol ? 8 : 0));
-            }
+        build_cones(N, be, T.cone, T.conek);
     }
     // element of each node's wall-condition gradients: among the incident
     // elements with a vertex on a wall edge the one of larger computational
