@@ -301,97 +301,286 @@ __global__ void k_fill_uniform(StateDev<S> st, int N, const double *consts, doub
     st.T[a] = (fld_t<S>)T;
 }
 
-// Full FP64 populations <-> stored deviations (internal order), one
-// population set per launch so that each half's kernel overlaps the other
-// half's host copy.  plane ([9 N]) and fields are in the caller's node
-// order: internal node a is caller node n2o[a].
-// part 0: the f plane; without fields, rho and u = sum (c_i + U) f_i / rho
-// go to tmp ([3 N], internal order, FP64).  part 1: the g plane, then the
-// fields (given, or T from sum g_i and tmp).
-template <class S>
-__global__ void k_import(StateDev<S> st, int N, const double *consts, const double *plane,
-                         const double *fields, int have_fields, double Cv, double Ux, double Uy,
-                         const int *n2o, double *tmp, int part)
+// ---------------------------------------------------------------------------
+// Exchange: full FP64 populations (or the FP32 form's stored deviations) <->
+// the stored form, internal order; the caller's arrays are in the caller's
+// node order (internal node a is caller node n2o[a]).
+//
+// Import was bound by the FP64 pipe (two lanes per SM and clock): about 70
+// operations per node and population set for the differences, sums, moments
+// and conversions (495 us for both sets at 2.0M nodes, 70 of HBM traffic; 192
+// us now, in one pass on the device exchange).  The
+// deviation forms now split and sum in 64-bit fixed point: a value below 2 is
+// q 2^-58, rounded once (3.5e-18 at most, half an FP64 ulp of 0.03), its
+// differences and sums are exact integers, and a difference is rounded to FP32
+// once.  About 30 FP64 operations are left per node for both sets.  A node with
+// a value outside that range (or not finite) takes the FP64 arithmetic.
+// ---------------------------------------------------------------------------
+constexpr int FIX_BITS = 58;
+constexpr double FIX_UNIT = 1.0 / (double)(1ll << FIX_BITS);
+
+// m 2^s, rounded to nearest (m < 2^53, s <= 35 and m 2^s < 2^60).
+__device__ __forceinline__ long long fix_shift(unsigned long long m, int s, bool neg)
 {
-    int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= N) return;
-    const int o = n2o[a];
-    double sum = 0, jx = 0, jy = 0;
-    for (int i = 0; i < NQ; ++i) {
-        const double v = plane[i * N + o];
-        pop_put1(st.post, i, a, N, part, v - consts[part * NQ + i]);
-        sum += v;
-        if (part == 0) {
-            jx += c_cx[i] * v;
-            jy += c_cy[i] * v;
+    if (s >= 0) {
+        m <<= s;
+    } else {
+        const int r = min(-s, 63);
+        m = (m + (1ull << (r - 1))) >> r;
+    }
+    return neg ? -(long long)m : (long long)m;
+}
+// v in units of 2^-FIX_BITS; false when v is not finite or |v| >= 2 (an FP32
+// deviation: 1).
+__device__ __forceinline__ bool to_fix(double v, long long &q)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)(b >> 52) & 0x7ff;
+    const unsigned long long m = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+    q = fix_shift(m, min(max(e, 1) - (1075 - FIX_BITS), 6), (long long)b < 0);
+    return e <= 1023;
+}
+__device__ __forceinline__ bool to_fix(float v, long long &q)
+{
+    const unsigned b = __float_as_uint(v);
+    const int e = (int)(b >> 23) & 0xff;
+    const unsigned long long m = (b & 0x7fffffu) | (e ? 1u << 23 : 0u);
+    q = fix_shift(m, min(max(e, 1) - (150 - FIX_BITS), 35), (int)b < 0);
+    return e <= 126; // |v| < 1: nine sums of a deviation and its reference stay below 2^63
+}
+// q 2^-FIX_BITS rounded to FP32: the upper 32 bits of |q| with the rest as a
+// sticky bit, through the 32-bit conversion.
+__device__ __forceinline__ float fix_to_float(long long q)
+{
+    const unsigned long long m = (unsigned long long)(q < 0 ? -q : q);
+    if (m == 0) return 0.f;
+    const int n = __clzll((long long)m);
+    const unsigned long long y = m << n;
+    const unsigned h = (unsigned)(y >> 32) | ((unsigned)y ? 1u : 0u);
+    const float f = __uint2float_rn(h) * __uint_as_float((unsigned)(127 + 32 - FIX_BITS - n) << 23);
+    return q < 0 ? -f : f;
+}
+
+// A stored value as FP64: by its bits (f2d_bits) where they are a normal
+// number, spared the FP64 pipe's conversion.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v)
+{
+    const unsigned m = __float_as_uint(v) & 0x7fffffffu;
+    return m - 0x00800000u < 0x7f000000u ? f2d_bits(v) : (double)v;
+}
+
+// A block's copies of the 18 reference populations and their fixed-point
+// values.
+struct RefTable {
+    double c[2 * NQ];
+    long long q[2 * NQ];
+    int ok;
+    __device__ void load(const double *consts)
+    {
+        bool in = true;
+        if (threadIdx.x < 2 * NQ) {
+            c[threadIdx.x] = consts[threadIdx.x];
+            in = to_fix(consts[threadIdx.x], q[threadIdx.x]);
+        }
+        const int all = __syncthreads_and(in);
+        if (threadIdx.x == 0) ok = all;
+        __syncthreads();
+    }
+};
+
+// sum, x and y sums over the lattice of the nine values of a node
+struct NodeSums {
+    double s, x, y;
+};
+template <class T> __device__ __forceinline__ void lattice_sums(const T v[NQ], T &s, T &x, T &y)
+{
+    s = v[0];
+#pragma unroll
+    for (int i = 1; i < NQ; ++i) s += v[i];
+    x = ((((v[1] - v[3]) + v[5]) - v[6]) - v[7]) + v[8];
+    y = ((((v[2] - v[4]) + v[5]) + v[6]) - v[7]) - v[8];
+}
+
+// The nine values of one set (part 0: f, 1: g) of a node: what is stored, and
+// the sums of the full populations.  V = double: full populations; V = float:
+// stored deviations.
+template <class S, class V>
+__device__ __forceinline__ NodeSums import_half(const RefTable &R, const V v[NQ], int part, fld_t<S> d[NQ])
+{
+    NodeSums r;
+    if constexpr (std::is_same<S, double>::value) { // no reference
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) d[i] = v[i];
+        lattice_sums(d, r.s, r.x, r.y);
+    } else {
+        long long q[NQ];
+        bool in = R.ok != 0;
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) in &= to_fix(v[i], q[i]);
+        if (in) {
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) {
+                const long long c = R.q[part * NQ + i];
+                if constexpr (std::is_same<V, double>::value) {
+                    d[i] = fix_to_float(q[i] - c);
+                } else {
+                    d[i] = v[i];
+                    q[i] += c;
+                }
+            }
+            long long s, x, y;
+            lattice_sums(q, s, x, y);
+            r.s = (double)s * FIX_UNIT;
+            r.x = (double)x * FIX_UNIT;
+            r.y = (double)y * FIX_UNIT;
+        } else {
+            double w[NQ];
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) {
+                const double c = R.c[part * NQ + i];
+                if constexpr (std::is_same<V, double>::value) {
+                    w[i] = v[i];
+                    d[i] = (float)(w[i] - c);
+                } else {
+                    w[i] = (double)v[i] + c;
+                    d[i] = v[i];
+                }
+            }
+            lattice_sums(w, r.s, r.x, r.y);
         }
     }
+    return r;
+}
+
+// rho and u = sum (c_i + U) f_i / rho from the f set's sums.
+__device__ __forceinline__ void import_velocity(const NodeSums &F, double Ux, double Uy, double &ux, double &uy)
+{
+    ux = F.x / F.s + Ux;
+    uy = F.y / F.s + Uy;
+}
+template <class S>
+__device__ __forceinline__ void import_fields(const StateDev<S> &st, int a, double rho, double ux, double uy, double sg,
+                                              double Cv)
+{
+    const double E = sg / (2 * rho);
+    st.rho[a] = (fld_t<S>)rho;
+    st.ux[a] = (fld_t<S>)ux;
+    st.uy[a] = (fld_t<S>)uy;
+    st.T[a] = (fld_t<S>)((E - 0.5 * (ux * ux + uy * uy)) / Cv);
+}
+
+// Host exchange, one population set per launch so that each half's kernel
+// overlaps the other half's host copy.  V = double: the full populations of
+// any form; V = float: the FP32 form's stored deviations, kept bit for bit.
+// part 0: the f plane; without fields, rho and u go to tmp ([3 N], internal
+// order, FP64).  part 1: the g plane, then the fields (given, or T from
+// sum g_i and tmp).  All loads of a node go out together.
+template <class S, class V>
+__global__ void __launch_bounds__(256) k_import(StateDev<S> st, int N, const double *__restrict__ consts,
+                                                const V *__restrict__ plane, const double *__restrict__ fields,
+                                                double Cv, double Ux, double Uy, const int *__restrict__ n2o,
+                                                double *tmp, int part)
+{
+    __shared__ RefTable R;
+    R.load(consts);
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= N) return;
+    const int o = n2o[a];
+    V v[NQ];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) v[i] = plane[(size_t)i * N + o];
+    fld_t<S> d[NQ];
+    const NodeSums n = import_half<S>(R, v, part, d);
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) pop_put1(st.post, i, a, N, part, d[i]);
     if (part == 0) {
-        if (!have_fields) {
-            tmp[a] = sum;
-            tmp[N + a] = jx / sum + Ux; // lattice c_i + U
-            tmp[2 * N + a] = jy / sum + Uy;
+        if (!fields) {
+            double ux, uy;
+            import_velocity(n, Ux, Uy, ux, uy);
+            tmp[a] = n.s;
+            tmp[N + a] = ux;
+            tmp[2 * N + a] = uy;
         }
-    } else if (have_fields) {
+    } else if (fields) {
         st.rho[a] = (fld_t<S>)fields[o];
         st.ux[a] = (fld_t<S>)fields[N + o];
         st.uy[a] = (fld_t<S>)fields[2 * N + o];
         st.T[a] = (fld_t<S>)fields[3 * N + o];
     } else {
-        const double r = tmp[a], ux = tmp[N + a], uy = tmp[2 * N + a], E = sum / (2 * r);
-        st.rho[a] = (fld_t<S>)r;
-        st.ux[a] = (fld_t<S>)ux;
-        st.uy[a] = (fld_t<S>)uy;
-        st.T[a] = (fld_t<S>)((E - 0.5 * (ux * ux + uy * uy)) / Cv);
+        import_fields(st, a, tmp[a], tmp[N + a], tmp[2 * N + a], n.s, Cv);
     }
 }
 
-// The FP32-deviation form's stored pairs <-> the caller's [9][N] FP32
-// planes of the same deviations, without conversion (the exchange is exact
-// both ways).  Import, part 0: the f plane, and rho and u into tmp from the
-// full FP64 populations d + ref, as k_import computes them; part 1: the g
-// plane and the fields.
-__global__ void k_import_stored(StateDev<float> st, int N, const double *consts, const float *plane, double Cv,
-                               double Ux, double Uy, const int *n2o, double *tmp, int part)
+// Device exchange: both sets in one pass, the pairs stored whole.
+template <class S>
+__global__ void __launch_bounds__(256) k_import_dev(StateDev<S> st, int N, const double *__restrict__ consts,
+                                                    const double *__restrict__ f, const double *__restrict__ g,
+                                                    double Cv, double Ux, double Uy, const int *__restrict__ n2o)
 {
-    int a = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ RefTable R;
+    R.load(consts);
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= N) return;
     const int o = n2o[a];
-    double sum = 0, jx = 0, jy = 0;
+    double v[NQ], w[NQ];
+#pragma unroll
     for (int i = 0; i < NQ; ++i) {
-        const float d = plane[i * N + o];
-        pop_put1(st.post, i, a, N, part, (double)d);
-        const double v = (double)d + consts[part * NQ + i];
-        sum += v;
-        if (part == 0) {
-            jx += c_cx[i] * v;
-            jy += c_cy[i] * v;
-        }
+        v[i] = f[(size_t)i * N + o];
+        w[i] = g[(size_t)i * N + o];
     }
-    if (part == 0) {
-        tmp[a] = sum;
-        tmp[N + a] = jx / sum + Ux;
-        tmp[2 * N + a] = jy / sum + Uy;
-    } else {
-        const double r = tmp[a], ux = tmp[N + a], uy = tmp[2 * N + a], E = sum / (2 * r);
-        st.rho[a] = (float)r;
-        st.ux[a] = (float)ux;
-        st.uy[a] = (float)uy;
-        st.T[a] = (float)((E - 0.5 * (ux * ux + uy * uy)) / Cv);
+    fld_t<S> df[NQ], dg[NQ];
+    const NodeSums F = import_half<S>(R, v, 0, df), G = import_half<S>(R, w, 1, dg);
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) fg_put(st.post, i, a, N, df[i], dg[i]);
+    double ux, uy;
+    import_velocity(F, Ux, Uy, ux, uy);
+    import_fields(st, a, F.s, ux, uy, G.s, Cv);
+}
+
+// The sets as full FP64 populations into the caller's planes, one set per grid
+// row and one plane at a time (2.0M nodes: 150 us with the loads of nine or
+// eighteen planes together ahead of their scattered stores).
+template <class S>
+__global__ void __launch_bounds__(256) k_export_dev(StateDev<S> st, int N, const double *consts, double *f, double *g,
+                                                    const int *n2o)
+{
+    const int a = blockIdx.x * blockDim.x + threadIdx.x, part = blockIdx.y;
+    if (a >= N) return;
+    const int o = n2o[a];
+    double *plane = part ? g : f;
+#pragma unroll 1
+    for (int i = 0; i < NQ; ++i) {
+        fld_t<S> x, y;
+        fg_get(st.post, i, a, N, x, y);
+        plane[(size_t)i * N + o] = widen(part ? y : x) + consts[part * NQ + i];
     }
+}
+template <class S>
+__global__ void k_fields_dev(StateDev<S> st, int N, double *rho, double *ux, double *uy, double *T,
+                             const int *__restrict__ n2o)
+{
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= N) return;
+    const int o = n2o[a];
+    if (rho) rho[o] = widen(st.rho[a]);
+    if (ux) ux[o] = widen(st.ux[a]);
+    if (uy) uy[o] = widen(st.uy[a]);
+    if (T) T[o] = widen(st.T[a]);
 }
 
 // Export: part 0 the f deviations, part 1 the g deviations.
-__global__ void k_export_stored(StateDev<float> st, int N, float *plane, const int *n2o, int part)
+__global__ void __launch_bounds__(256) k_export_stored(StateDev<float> st, int N, float *plane,
+                                                       const int *__restrict__ n2o, int part)
 {
-    int a = blockIdx.x * blockDim.x + threadIdx.x;
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= N) return;
     const int o = n2o[a];
-    for (int i = 0; i < NQ; ++i) {
-        float f, g;
-        fg_get(st.post, i, a, N, f, g);
-        plane[i * N + o] = part == 0 ? f : g;
-    }
+    float v[NQ];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) v[i] = st.post[2 * ((size_t)i * N + a) + part];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) plane[(size_t)i * N + o] = v[i];
 }
 
 // part 0: the f plane into plane; part 1: the g plane (plane may be
@@ -866,15 +1055,17 @@ cudaError_t alelb::import_enqueue(alelb_solver *s, const double *f, const double
     if (st != cudaSuccess) return st;
     const dim3 grid((N + 255) / 256), block(256);
     with_state(s, [&](auto &sx, auto &) {
-        k_import<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, s->d_scratch, dfields, have, s->Cv, s->U[0],
-                                                s->U[1], s->mesh->d_n2o, dfields, 0);
+        k_import<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, (const double *)s->d_scratch,
+                                                (const double *)(have ? dfields : nullptr), s->Cv, s->U[0], s->U[1],
+                                                s->mesh->d_n2o, dfields, 0);
     });
     st = cudaGetLastError();
     if (st == cudaSuccess) st = cudaStreamWaitEvent(s->stream, s->ev_copy[1], 0);
     if (st == cudaSuccess)
         with_state(s, [&](auto &sx, auto &) {
-            k_import<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, s->d_scratch + (size_t)9 * N, dfields,
-                                                    have, s->Cv, s->U[0], s->U[1], s->mesh->d_n2o, dfields, 1);
+            k_import<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, (const double *)(s->d_scratch + (size_t)9 * N),
+                                                    (const double *)(have ? dfields : nullptr), s->Cv, s->U[0], s->U[1],
+                                                    s->mesh->d_n2o, dfields, 1);
         });
     if (st == cudaSuccess) st = cudaGetLastError();
     return st;
@@ -919,13 +1110,13 @@ cudaError_t alelb::import_stored_enqueue(alelb_solver *s, const float *f, const 
     if (st == cudaSuccess) st = cudaEventRecord(s->ev_copy[1], s->copy_stream);
     if (st != cudaSuccess) return st;
     const dim3 grid((N + 255) / 256), block(256);
-    k_import_stored<<<grid, block, 0, s->stream>>>(s->sf, N, s->d_consts, pf, s->Cv, s->U[0], s->U[1],
-                                                  s->mesh->d_n2o, tmp, 0);
+    k_import<<<grid, block, 0, s->stream>>>(s->sf, N, s->d_consts, (const float *)pf, (const double *)nullptr, s->Cv,
+                                            s->U[0], s->U[1], s->mesh->d_n2o, tmp, 0);
     st = cudaGetLastError();
     if (st == cudaSuccess) st = cudaStreamWaitEvent(s->stream, s->ev_copy[1], 0);
     if (st == cudaSuccess) {
-        k_import_stored<<<grid, block, 0, s->stream>>>(s->sf, N, s->d_consts, pg, s->Cv, s->U[0], s->U[1],
-                                                      s->mesh->d_n2o, tmp, 1);
+        k_import<<<grid, block, 0, s->stream>>>(s->sf, N, s->d_consts, (const float *)pg, (const double *)nullptr, s->Cv,
+                                                s->U[0], s->U[1], s->mesh->d_n2o, tmp, 1);
         st = cudaGetLastError();
     }
     return st;
@@ -982,8 +1173,7 @@ extern "C" alelb_status alelb_get_pops_dev(alelb_solver *s, double *f, double *g
     const int N = m->T.N;
     const dim3 grid((N + 255) / 256), block(256);
     with_state(s, [&](auto &sx, auto &) {
-        k_export<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, f, nullptr, m->d_n2o, 0);
-        k_export<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, g, nullptr, m->d_n2o, 1);
+        k_export_dev<<<dim3(grid.x, 2), block, 0, s->stream>>>(sx, N, s->d_consts, f, g, m->d_n2o);
     });
     const cudaError_t st = cudaGetLastError();
     if (st != cudaSuccess) return cuda_fail(s, st);
@@ -995,13 +1185,9 @@ extern "C" alelb_status alelb_set_pops_dev(alelb_solver *s, const double *f, con
     if (!s || !f || !g) return ALELB_ERR_ARG;
     if (!on_mesh_device(s, f, "set_pops_dev") || !on_mesh_device(s, g, "set_pops_dev")) return ALELB_ERR_ARG;
     const int N = s->mesh->T.N;
-    double *tmp = s->d_scratch + (size_t)18 * N;
     const dim3 grid((N + 255) / 256), block(256);
     with_state(s, [&](auto &sx, auto &) {
-        k_import<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, f, nullptr, 0, s->Cv, s->U[0], s->U[1],
-                                                s->mesh->d_n2o, tmp, 0);
-        k_import<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, g, nullptr, 0, s->Cv, s->U[0], s->U[1],
-                                                s->mesh->d_n2o, tmp, 1);
+        k_import_dev<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, f, g, s->Cv, s->U[0], s->U[1], s->mesh->d_n2o);
     });
     cudaError_t st = cudaGetLastError();
     if (st == cudaSuccess) st = cudaStreamSynchronize(s->stream);
@@ -1013,20 +1199,14 @@ extern "C" alelb_status alelb_set_pops_dev(alelb_solver *s, const double *f, con
 extern "C" alelb_status alelb_moments_dev(alelb_solver *s, double *rho, double *ux, double *uy, double *T)
 {
     if (!s) return ALELB_ERR_ARG;
-    double *const out[4] = {rho, ux, uy, T};
-    for (double *p : out)
+    for (double *p : {rho, ux, uy, T})
         if (p && !on_mesh_device(s, p, "moments_dev")) return ALELB_ERR_ARG;
     alelb_mesh *m = s->mesh;
     const int N = m->T.N;
-    double *dfields = s->d_scratch + (size_t)18 * N;
     with_state(s, [&](auto &sx, auto &) {
-        k_export<<<(N + 255) / 256, 256, 0, s->stream>>>(sx, N, s->d_consts, nullptr, dfields, m->d_n2o, 1);
+        k_fields_dev<<<(N + 255) / 256, 256, 0, s->stream>>>(sx, N, rho, ux, uy, T, m->d_n2o);
     });
-    cudaError_t st = cudaGetLastError();
-    for (int c = 0; c < 4 && st == cudaSuccess; ++c)
-        if (out[c])
-            st = cudaMemcpyAsync(out[c], dfields + (size_t)c * N, (size_t)N * sizeof(double), cudaMemcpyDeviceToDevice,
-                                 s->stream);
+    const cudaError_t st = cudaGetLastError();
     if (st != cudaSuccess) return cuda_fail(s, st);
     return alelb_sync(s);
 }

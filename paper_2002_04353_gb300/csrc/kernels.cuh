@@ -97,19 +97,19 @@ template <class A> __device__ __forceinline__ void fg_put(__half *p, int i, int 
 }
 // One half of the pair: part 0 writes f_i, part 1 writes g_i (rounded as
 // fg_put rounds it).
-__device__ __forceinline__ void pop_put1(double *p, int i, int x, int N, int part, double v)
+template <class A> __device__ __forceinline__ void pop_put1(double *p, int i, int x, int N, int part, A v)
 {
-    p[(part * NQ + i) * N + x] = v;
+    p[(part * NQ + i) * N + x] = (double)v;
 }
-__device__ __forceinline__ void pop_put1(float *p, int i, int x, int N, int part, double v)
+template <class A> __device__ __forceinline__ void pop_put1(float *p, int i, int x, int N, int part, A v)
 {
     p[2 * (i * N + x) + part] = (float)v;
 }
-__device__ __forceinline__ void pop_put1(__nv_bfloat16 *p, int i, int x, int N, int part, double v)
+template <class A> __device__ __forceinline__ void pop_put1(__nv_bfloat16 *p, int i, int x, int N, int part, A v)
 {
     p[2 * (i * N + x) + part] = __float2bfloat16_rn((float)v);
 }
-__device__ __forceinline__ void pop_put1(__half *p, int i, int x, int N, int part, double v)
+template <class A> __device__ __forceinline__ void pop_put1(__half *p, int i, int x, int N, int part, A v)
 {
     p[2 * (i * N + x) + part] = __float2half_rn((float)v * FP16_DEV_SCALE);
 }
