@@ -1220,8 +1220,9 @@ extern "C" alelb_status alelb_forces(alelb_solver *s, double out[6])
         quad_forces(s, sc);
     } else if (m->nw > 0) {
         with_state(s, [&](auto &sx, auto &) {
-            k_forces<<<1, 256, 0, s->stream>>>(m->dev, m->mst, sc, sx, m->d_wedges, m->nw, s->mu, s->Cv,
-                                               s->d_out);
+            k_forces<<<force_blocks(m->nw), FORCE_BS, 0, s->stream>>>(m->dev, m->mst, sc, sx, m->d_wedges, m->nw, s->mu,
+                                                                      s->Cv, s->d_scratch);
+            k_forces_sum<<<1, 128, 0, s->stream>>>(s->d_scratch, force_blocks(m->nw), s->d_out);
         });
     } else {
         cudaMemsetAsync(s->d_out, 0, 4 * sizeof(double), s->stream);

@@ -1379,57 +1379,85 @@ static __global__ void k_locate(MeshDev M, MapStatic MS, MapScalars sc, MapScala
     }
 }
 
-// Wall forces: one block, fixed-order FP64 reduction.
+// Wall forces: Simpson's rule on the wall edges, one thread per node of an
+// edge (item 3 edge + place), each block's sums in part[4 block ..], then one
+// block over the rows: every sum in a fixed order.  Bound by the FP64 pipe of
+// the SMs it runs on (some 350 operations per item), so the items are spread
+// over many small blocks; in one block of 256 it took 52 us with 320 edges.
 // out = {Fx_p, Fy_p, Fx_v, Fy_v}.
-template <class S>
-__global__ void __launch_bounds__(256) k_forces(MeshDev M, MapStatic MS, MapScalars sc,
-                                                StateDev<S> st, const int2 *wedges, int nw,
-                                                double mu, double Cv, double *out)
+constexpr int FORCE_BS = 64;
+inline int force_blocks(int nw) { return (3 * nw + FORCE_BS - 1) / FORCE_BS; }
+
+// The contribution of a node: weight wgt, outward normal n, pressure rho T,
+// velocity gradients d.
+__device__ __forceinline__ void force_item(double wgt, double nx, double ny, double rho, double T, const double d[4],
+                                           double mu, double Cv, double acc[4])
 {
-    __shared__ double red[4][256];
-    double acc[4] = {0, 0, 0, 0};
-    for (int w = threadIdx.x; w < nw; w += blockDim.x) {
-        int e = wedges[w].x, k = wedges[w].y, k1 = (k + 1) % 3;
-        int nodes[3] = {M.conn[6 * e + k], M.conn[6 * e + 3 + k], M.conn[6 * e + k1]};
-        double2 A0 = M.X[nodes[0]], B0 = M.X[nodes[2]];
-        double xa, ya, xb, yb;
-        map_position(MS, sc, nodes[0], A0.x, A0.y, xa, ya);
-        map_position(MS, sc, nodes[2], B0.x, B0.y, xb, yb);
-        double tx = xb - xa, ty = yb - ya, L = sqrt(tx * tx + ty * ty);
-        double nx = -ty / L, ny = tx / L; // out of the body, into the fluid
-        double wgt[3] = {L / 6.0, 4.0 * L / 6.0, L / 6.0};
-        for (int j = 0; j < 3; ++j) {
-            int a = nodes[j];
-            double2 Xa = M.X[a];
-            double xX, xY, yX, yY, Vx, Vy, a11, a12, a21, a22;
-            map_node(MS, sc, a, Xa.x, Xa.y, xX, xY, yX, yY, Vx, Vy);
-            metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
-            double KX, KY, d[4];
-            owner_grad(M, a, st.ux, KX, KY);
-            d[0] = a11 * KX + a21 * KY;
-            d[1] = a12 * KX + a22 * KY;
-            owner_grad(M, a, st.uy, KX, KY);
-            d[2] = a11 * KX + a21 * KY;
-            d[3] = a12 * KX + a22 * KY;
-            double div = d[0] + d[3];
-            double p = (double)st.rho[a] * (double)st.T[a];
-            double txx = mu * (2.0 * d[0] - div / Cv);
-            double tyy = mu * (2.0 * d[3] - div / Cv);
-            double txy = mu * (d[1] + d[2]);
-            acc[0] += wgt[j] * (-p * nx);
-            acc[1] += wgt[j] * (-p * ny);
-            acc[2] += wgt[j] * (txx * nx + txy * ny);
-            acc[3] += wgt[j] * (txy * nx + tyy * ny);
-        }
-    }
-    for (int c = 0; c < 4; ++c) red[c][threadIdx.x] = acc[c];
+    const double div = d[0] + d[3], p = rho * T;
+    const double txx = mu * (2.0 * d[0] - div / Cv);
+    const double tyy = mu * (2.0 * d[3] - div / Cv);
+    const double txy = mu * (d[1] + d[2]);
+    acc[0] = wgt * (-p * nx);
+    acc[1] = wgt * (-p * ny);
+    acc[2] = wgt * (txx * nx + txy * ny);
+    acc[3] = wgt * (txy * nx + tyy * ny);
+}
+
+__device__ __forceinline__ void force_block_sums(double acc[4], double *part)
+{
+    __shared__ double red[FORCE_BS / 32][4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+    if ((threadIdx.x & 31) == 0)
+        for (int c = 0; c < 4; ++c) red[threadIdx.x >> 5][c] = acc[c];
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
-            for (int c = 0; c < 4; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + s];
-        __syncthreads();
+    if (threadIdx.x < 4) {
+        double v = red[0][threadIdx.x];
+        for (int w = 1; w < FORCE_BS / 32; ++w) v += red[w][threadIdx.x];
+        part[4 * (size_t)blockIdx.x + threadIdx.x] = v;
     }
-    if (threadIdx.x < 4) out[threadIdx.x] = red[threadIdx.x][0];
+}
+
+// One warp per component.
+static __global__ void __launch_bounds__(128) k_forces_sum(const double *part, int rows, double *out)
+{
+    const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double v = 0.0;
+    for (int r = lane; r < rows; r += 32) v += part[4 * (size_t)r + c];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) out[c] = v;
+}
+
+template <class S>
+__global__ void __launch_bounds__(FORCE_BS) k_forces(MeshDev M, MapStatic MS, MapScalars sc, StateDev<S> st,
+                                                     const int2 *wedges, int nw, double mu, double Cv, double *part)
+{
+    double acc[4] = {0, 0, 0, 0};
+    const int t = blockIdx.x * FORCE_BS + threadIdx.x;
+    if (t < 3 * nw) {
+        const int w = t / 3, j = t % 3, e = wedges[w].x, k = wedges[w].y, k1 = (k + 1) % 3;
+        const int n0 = M.conn[6 * e + k], n2 = M.conn[6 * e + k1];
+        const int a = j == 0 ? n0 : j == 1 ? M.conn[6 * e + 3 + k] : n2;
+        const double2 A0 = M.X[n0], B0 = M.X[n2], Xa = M.X[a];
+        double xa, ya, xb, yb;
+        map_position(MS, sc, n0, A0.x, A0.y, xa, ya);
+        map_position(MS, sc, n2, B0.x, B0.y, xb, yb);
+        const double tx = xb - xa, ty = yb - ya, L = sqrt(tx * tx + ty * ty);
+        const double nx = -ty / L, ny = tx / L; // out of the body, into the fluid
+        double xX, xY, yX, yY, Vx, Vy, a11, a12, a21, a22;
+        map_node(MS, sc, a, Xa.x, Xa.y, xX, xY, yX, yY, Vx, Vy);
+        metric_inverse_T(xX, xY, yX, yY, a11, a12, a21, a22);
+        double KX, KY, d[4];
+        owner_grad(M, a, st.ux, KX, KY);
+        d[0] = a11 * KX + a21 * KY;
+        d[1] = a12 * KX + a22 * KY;
+        owner_grad(M, a, st.uy, KX, KY);
+        d[2] = a11 * KX + a21 * KY;
+        d[3] = a12 * KX + a22 * KY;
+        force_item(j == 1 ? 4.0 * L / 6.0 : L / 6.0, nx, ny, (double)st.rho[a], (double)st.T[a], d, mu, Cv, acc);
+    }
+    force_block_sums(acc, part);
 }
 
 // det g > 0 check at every node (alelb_mesh_move).
