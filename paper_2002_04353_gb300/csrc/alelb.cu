@@ -664,6 +664,7 @@ cudaError_t launch_step(alelb_solver *s, const StateDev<S> &st0, KinParams<A> &K
                            : (s->flags & ALELB_FLAG_MIDPOINT) ? solver_map(s, map_scalars(m->T.mkind, m->T.mp, s->t + 0.5))
                                                               : sc;
     const MapScalarsF sfd = to_f32(scd, m->T);
+    const DepTab dep = dep_table(scd);
     // The two passes in every form; the FP64 form keeps the plain pass where
     // no FP32 certificate covers the departure point, so that nothing would
     // settle in the first one.
@@ -729,24 +730,24 @@ cudaError_t launch_step(alelb_solver *s, const StateDev<S> &st0, KinParams<A> &K
                 // where threads are few (1k box: 10, 17, 34; equal at 9k).
                 const dim3 gb(FAST_BS), g1((N + FAST_BS - 1) / FAST_BS, NQ), g3(g1.x, NQ / 3), g9(g1.x, 1);
                 if (m->T.mkind == MK_NONE || m->T.mkind == MK_PLUNGE)
-                    launch_pdl(k_stream_fast<S, A, 1, true>, g1, gb, s->stream, m->dev, m->mst, scd, sfd, K, st);
+                    launch_pdl(k_stream_fast<S, A, 1, true>, g1, gb, s->stream, m->dev, m->mst, scd, sfd, K, st, dep);
                 else if (N < FAST64_G3_NODES)
-                    launch_pdl(k_stream_fast<S, A, 1, false>, g1, gb, s->stream, m->dev, m->mst, scd, sfd, K, st);
+                    launch_pdl(k_stream_fast<S, A, 1, false>, g1, gb, s->stream, m->dev, m->mst, scd, sfd, K, st, dep);
                 else if (N < FAST64_G9_NODES)
-                    launch_pdl(k_stream_fast<S, A, 3, false>, g3, gb, s->stream, m->dev, m->mst, scd, sfd, K, st);
+                    launch_pdl(k_stream_fast<S, A, 3, false>, g3, gb, s->stream, m->dev, m->mst, scd, sfd, K, st, dep);
                 else
-                    launch_pdl(k_stream_fast<S, A, NQ, false>, g9, gb, s->stream, m->dev, m->mst, scd, sfd, K, st);
+                    launch_pdl(k_stream_fast<S, A, NQ, false>, g9, gb, s->stream, m->dev, m->mst, scd, sfd, K, st, dep);
                 break;
             }
             if (m->T.mkind == MK_NONE || m->T.mkind == MK_PLUNGE)
                 launch_pdl(k_stream_fast<S, A, FAST_G, true>, dim3((N + FAST_BS - 1) / FAST_BS, NQ / FAST_G),
-                           dim3(FAST_BS), s->stream, m->dev, m->mst, scd, sfd, K, st);
+                           dim3(FAST_BS), s->stream, m->dev, m->mst, scd, sfd, K, st, dep);
             else if (N < FAST_G_NODES)
                 launch_pdl(k_stream_fast<S, A, FAST_G, false>, dim3((N + FAST_BS - 1) / FAST_BS, NQ / FAST_G),
-                           dim3(FAST_BS), s->stream, m->dev, m->mst, scd, sfd, K, st);
+                           dim3(FAST_BS), s->stream, m->dev, m->mst, scd, sfd, K, st, dep);
             else
                 launch_pdl(k_stream_fast<S, A, NQ, false>, dim3((N + FAST_BS - 1) / FAST_BS, 1), dim3(FAST_BS),
-                           s->stream, m->dev, m->mst, scd, sfd, K, st);
+                           s->stream, m->dev, m->mst, scd, sfd, K, st, dep);
             break;
         case KT_SLOW: {
             // every block resident at once: the list is spread over all

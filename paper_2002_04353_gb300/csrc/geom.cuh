@@ -120,6 +120,16 @@ __device__ __forceinline__ double f2d_bits(float v)
     return __hiloint2double((int)hi, (int)(m >= 0x00800000u ? b << 29 : 0u));
 }
 
+// v 2^k by the exponent field (|k| <= 2), off the FP64 pipe: exact for zero
+// and numbers well inside the range, others are returned unscaled (they occur
+// as shape-function factors below 1e-300 only).
+__device__ __forceinline__ double scale2_bits(double v, int k)
+{
+    const int hi = __double2hiint(v);
+    const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+    return __hiloint2double(e - 8u < 2032u ? hi + (k << 20) : hi, __double2loint(v));
+}
+
 // Metrics x_X, x_Y, y_X, y_Y and mesh velocity V_G at a node.
 ALELB_HD __forceinline__ void map_node(const MapStatic &M, const MapScalars &S, int a,
                                          double X, double Y, double &xX, double &xY,

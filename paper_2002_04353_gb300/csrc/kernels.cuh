@@ -385,6 +385,19 @@ __device__ __forceinline__ double lattice_sum(double a, double b, int cx, int cy
     return cx == 0 ? (cy == 0 ? 0.0 : v) : (cy == 0 ? u : da(u, v));
 }
 
+// On a translation c_i - w is the same at every node: formed on the host, by
+// the operations of departure64<true>.
+struct DepTab {
+    double2 c[NQ];
+};
+inline DepTab dep_table(const MapScalars &sc)
+{
+    DepTab D;
+    const double wx = 0.0 - sc.Ux, wy = sc.vy - sc.Uy;
+    for (int i = 0; i < NQ; ++i) D.c[i] = make_double2((double)lat_cx(i) - wx, (double)lat_cy(i) - wy);
+    return D;
+}
+
 // The canonical departure point (departure() in geom.cuh) of population i.
 template <bool TR>
 __device__ __forceinline__ void departure64(const Node64 &n, int i, double2 X, double &px, double &py)
@@ -414,10 +427,12 @@ __device__ __forceinline__ void interp64(const MeshDev &M, const double *post, i
     if (sy) v0.y = da(v0.y, sy * M.Ly);
     const double dx = ds(px, v0.x), dy = ds(py, v0.y);
     const double xi = dfma(j1.x, dx, dm(j1.y, dy)), eta = dfma(j2.x, dx, dm(j2.y, dy));
+    // l (2 l - 1) = l - 2 l (the other two), the edges' products shared: 11
+    // operations for the six weights
     const double l0 = ds(ds(1.0, xi), eta);
-    const double q = dm(4.0, xi), r = dm(4.0, eta);
-    const double w[6] = {dm(l0, dfma(2.0, l0, -1.0)), dm(xi, dfma(2.0, xi, -1.0)), dm(eta, dfma(2.0, eta, -1.0)),
-                         dm(q, l0), dm(q, eta), dm(r, l0)};
+    const double A = dm(xi, l0), B = dm(xi, eta), C = dm(eta, l0);
+    const double w[6] = {dfma(-2.0, da(A, C), l0), dfma(-2.0, da(A, B), xi), dfma(-2.0, da(B, C), eta),
+                         scale2_bits(A, 2), scale2_bits(B, 2), scale2_bits(C, 2)};
     double fb, gb;
     fg_get(post, i, nb[0], N, fb, gb);
     f = dm(w[0], fb);
@@ -763,12 +778,15 @@ static_assert(NQ % FAST_G == 0 && NQ % BATCH_FAST_G == 0, "directions per thread
 // deviation forms' certified FP32 one (the previous-step element, else the
 // exterior cone), the departure point and the interpolation of an accepted
 // population run in FP64 (codes as stream_fast_pop's).  Bound by the FP64
-// pipe (two lanes per SM and clock): 36 FP64 operations per population, so
-// the element search and its predicates stay off that pipe.
+// pipe (two lanes per SM and clock): 31 FP64 operations per population on a
+// translation (150,400 nodes: 80 us; 99 at 42, with c_i - w formed per thread
+// and every weight by itself), so the element search and its predicates stay
+// off that pipe.
 template <int G, bool TR>
 __device__ __forceinline__ void stream_fast_pops64(const MeshDev &M, const MapStatic &MS, const MapScalars &sc,
                                                    const MapScalarsF &sf, const KinParams<double> &K,
-                                                   const StateDev<double> &st, int a, int i0, int code[G])
+                                                   const StateDev<double> &st, int a, int i0, int code[G],
+                                                   const DepTab *D)
 {
     const int N = M.N;
     int c[G];
@@ -779,7 +797,8 @@ __device__ __forceinline__ void stream_fast_pops64(const MeshDev &M, const MapSt
     const double2 X = M.X[a];
     FastMap F = TR ? fast_map_translation(sf, Xf) : fast_map(MS, sf, a, Xf);
     if (K.flags & (FLAG_LITERAL_VG | FLAG_EXACT_CHAR)) F.ok = false;
-    const Node64 n = node64<TR>(MS, sc, a, X, false);
+    Node64 n;
+    if (!TR) n = node64<TR>(MS, sc, a, X, false);
     if (!TR && i0 == 0 && st.met) { // for the derivative passes
         st.met[2 * a] = make_double2(n.a11, n.a12);
         st.met[2 * a + 1] = make_double2(n.a21, n.a22);
@@ -800,7 +819,13 @@ __device__ __forceinline__ void stream_fast_pops64(const MeshDev &M, const MapSt
         float xi, eta;
         if (fast_decide(M, F, Xf, bd, a, i, c[j], e, xi, eta)) {
             double px, py, f, g;
-            departure64<TR>(n, i, X, px, py);
+            if (TR) {
+                const double2 c = D->c[i];
+                px = ds(X.x, c.x);
+                py = ds(X.y, c.y);
+            } else {
+                departure64<TR>(n, i, X, px, py);
+            }
             interp64(M, st.post, N, i, e, 0, 0, px, py, f, g);
             fg_put(st.str, i, a, N, f, g);
             code[j] = 0;
@@ -818,14 +843,14 @@ __device__ __forceinline__ void stream_fast_pops64(const MeshDev &M, const MapSt
 template <int G, class S, class A, bool TR = false>
 __device__ __forceinline__ void stream_fast_group(const MeshDev &M, const MapStatic &MS, const MapScalars &sc,
                                                   const MapScalarsF &sf, const KinParams<A> &K,
-                                                  const StateDev<S> &st, int a)
+                                                  const StateDev<S> &st, int a, const DepTab *D = nullptr)
 {
     const int i0 = G * blockIdx.y;
     int code[G];
 #pragma unroll
     for (int j = 0; j < G; ++j) code[j] = 0;
     if constexpr (std::is_same<S, double>::value) {
-        if (a < M.N) stream_fast_pops64<G, TR>(M, MS, sc, sf, K, st, a, i0, code);
+        if (a < M.N) stream_fast_pops64<G, TR>(M, MS, sc, sf, K, st, a, i0, code, D);
     } else if (a < M.N) {
         // the loads of the thread's cache entries go out together (the
         // stores of the populations would otherwise order them one by one)
@@ -860,10 +885,10 @@ constexpr int FAST_BS = ALELB_FAST_BS;
 // translation (no map, plunge).
 template <class S, class A, int G, bool TR>
 __global__ void __launch_bounds__(FAST_BS) k_stream_fast(MeshDev M, MapStatic MS, MapScalars sc, MapScalarsF sf,
-                                                     KinParams<A> K, StateDev<S> st)
+                                                     KinParams<A> K, StateDev<S> st, const __grid_constant__ DepTab D)
 {
     wait_prior_grid();
-    stream_fast_group<G, S, A, TR>(M, MS, sc, sf, K, st, blockIdx.x * blockDim.x + threadIdx.x);
+    stream_fast_group<G, S, A, TR>(M, MS, sc, sf, K, st, blockIdx.x * blockDim.x + threadIdx.x, &D);
 }
 
 // One listed population (code = 9 node + direction): exact decision, then

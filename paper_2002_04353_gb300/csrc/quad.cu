@@ -56,7 +56,8 @@ __device__ __forceinline__ bool quad_fast_pop(const QuadDev &M, const FastMap &F
 // point, local coordinates and interpolation in FP64.
 template <bool TR>
 __device__ __forceinline__ bool quad_fast_pop64(const QuadDev &M, const FastMap &F, const Node64 &n, float4 Xf, double2 X,
-                                                const StateDev<double> &st, int a, int i, int c, unsigned lanes)
+                                                const StateDev<double> &st, int a, int i, int c, unsigned lanes,
+                                                const DepTab &D)
 {
     int e = 0;
     float cw[8];
@@ -64,7 +65,13 @@ __device__ __forceinline__ bool quad_fast_pop64(const QuadDev &M, const FastMap 
     bool in = quad_fast_decide(M, F, Xf, a, i, c, e, cw);
     __syncwarp(lanes);
     if (in) {
-        departure64<TR>(n, i, X, px, py);
+        if (TR) {
+            const double2 cw = D.c[i];
+            px = ds(X.x, cw.x);
+            py = ds(X.y, cw.y);
+        } else {
+            departure64<TR>(n, i, X, px, py);
+        }
         in = quad_local64(M, e, 0, 0, px, py, xi, eta);
     }
     __syncwarp(lanes);
@@ -335,7 +342,8 @@ __global__ void __launch_bounds__(128) kq_stream(QuadDev M, MapStatic MS, MapSca
 // 16 blocks an SM (35 us at 40).
 template <class S, class A, int G, bool TR>
 __global__ void __launch_bounds__(128, std::is_same<S, double>::value ? 1 : 16) kq_fast(QuadDev M, MapStatic MS, MapScalars scd, MapScalarsF sfd,
-                                               KinParams<A> K, StateDev<S> st, unsigned long long *stats)
+                                               KinParams<A> K, StateDev<S> st, unsigned long long *stats,
+                                               const __grid_constant__ DepTab D)
 {
     constexpr bool FP64 = std::is_same<S, double>::value;
     wait_prior_grid();
@@ -353,7 +361,7 @@ __global__ void __launch_bounds__(128, std::is_same<S, double>::value ? 1 : 16) 
         int c[G];
         if constexpr (FP64) {
             X = M.X[a];
-            n = node64<TR>(MS, scd, a, X, false);
+            if (!TR) n = node64<TR>(MS, scd, a, X, false);
             if (!TR && i0 == 0 && st.met) { // for the derivative passes
                 st.met[2 * a] = make_double2(n.a11, n.a12);
                 st.met[2 * a + 1] = make_double2(n.a21, n.a22);
@@ -367,7 +375,7 @@ __global__ void __launch_bounds__(128, std::is_same<S, double>::value ? 1 : 16) 
             __syncwarp(lanes);
             // (a node of zero mesh velocity fails the test: its c^_0 is zero)
             bool done;
-            if constexpr (FP64) done = quad_fast_pop64<TR>(M, F, n, Xf, X, st, a, i, c[j], lanes);
+            if constexpr (FP64) done = quad_fast_pop64<TR>(M, F, n, Xf, X, st, a, i, c[j], lanes, D);
             else done = quad_fast_pop<S, A>(M, F, Xf, st, a, i, lanes);
             if (!done && F.ok) {
                 const int ck = cone_missing(M, F, a, i);
@@ -664,10 +672,11 @@ cudaError_t quad_launch(alelb_solver *s, int kernel, const MapScalars &sc, const
         }
         case KT_FAST: {
             const MapScalarsF sfd = to_f32(scd, m->T);
+            const DepTab dep = dep_table(scd);
             const bool tr = m->T.mkind == MK_NONE || m->T.mkind == MK_PLUNGE;
             const dim3 gb(128), g1((N + 127) / 128, NQ), g3(g1.x, NQ / 3);
             if (tr) {
-                launch_pdl(kq_fast<S, A, 1, true>, g1, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st, s->d_stats);
+                launch_pdl(kq_fast<S, A, 1, true>, g1, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st, s->d_stats, dep);
                 break;
             }
             if constexpr (std::is_same<S, double>::value) {
@@ -676,11 +685,11 @@ cudaError_t quad_launch(alelb_solver *s, int kernel, const MapScalars &sc, const
                 // per thread; 160k box 280, 318, 326; 24k 54, 62, 80), one per
                 // direction below (1k box: 13, 24, 58 us)
                 if (N >= FAST64_G3_NODES) {
-                    launch_pdl(kq_fast<S, A, 3, false>, g3, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st, s->d_stats);
+                    launch_pdl(kq_fast<S, A, 3, false>, g3, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st, s->d_stats, dep);
                     break;
                 }
             }
-            launch_pdl(kq_fast<S, A, 1, false>, g1, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st, s->d_stats);
+            launch_pdl(kq_fast<S, A, 1, false>, g1, gb, s->stream, m->qdev, m->mst, scd, sfd, K, st, s->d_stats, dep);
             break;
         }
         case KT_SLOW: {

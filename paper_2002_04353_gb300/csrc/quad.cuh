@@ -575,16 +575,18 @@ __device__ __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, in
 // The pair (f_i, g_i) of the FP64 form interpolated at (xi, eta) of element
 // e: the nine shape functions are products of one-dimensional ones, so three
 // sums along xi and one along eta (24 operations of the FP64 pipe for the two
-// fields, against 27 for nine weights and their sums).
+// fields, against 27 for nine weights and their sums); the one-dimensional
+// functions are (xi^2 -+ xi)/2 and 1 - xi^2, four operations each direction.
 __device__ __forceinline__ void quad_interp64(const QuadDev &M, const double *post, int N, int i, int e, double xi,
                                               double eta, double &f, double &g)
 {
     int nb[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) nb[k] = M.conn[9 * e + k];
-    const double hx = dm(0.5, xi), hy = dm(0.5, eta);
-    const double lx[3] = {dm(hx, ds(xi, 1.0)), dfma(-xi, xi, 1.0), dm(hx, da(xi, 1.0))};
-    const double ly[3] = {dm(hy, ds(eta, 1.0)), dfma(-eta, eta, 1.0), dm(hy, da(eta, 1.0))};
+    const double hx = scale2_bits(xi, -1), hy = scale2_bits(eta, -1), x2 = dm(xi, xi), y2 = dm(eta, eta);
+    const double sx = scale2_bits(x2, -1), sy = scale2_bits(y2, -1);
+    const double lx[3] = {ds(sx, hx), ds(1.0, x2), da(sx, hx)};
+    const double ly[3] = {ds(sy, hy), ds(1.0, y2), da(sy, hy)};
     constexpr int at[3][3] = {{0, 4, 1}, {7, 8, 5}, {3, 6, 2}}; // local node at (i, j), row j along xi
     f = 0.0;
     g = 0.0;
