@@ -691,6 +691,8 @@ cudaError_t launch_step(alelb_solver *s, const StateDev<S> &st0, KinParams<A> &K
         }
         return cudaGetLastError();
     }
+    // one thread per node of a large mesh also takes the node's moments
+    const bool fused = std::is_same<S, float>::value && m->T.mkind != MK_NONE && m->T.mkind != MK_PLUNGE && N >= FAST_G_NODES;
     int seq[KT_N], ns = 0;
     if (passes) {
         seq[ns++] = KT_FAST;
@@ -745,6 +747,9 @@ cudaError_t launch_step(alelb_solver *s, const StateDev<S> &st0, KinParams<A> &K
             else if (N < FAST_G_NODES)
                 launch_pdl(k_stream_fast<S, A, FAST_G, false>, dim3((N + FAST_BS - 1) / FAST_BS, NQ / FAST_G),
                            dim3(FAST_BS), s->stream, m->dev, m->mst, scd, sfd, K, st, dep);
+            else if constexpr (std::is_same<S, float>::value)
+                launch_pdl(k_stream_fast_moments<FAST_BS>, dim3((N + FAST_BS - 1) / FAST_BS), dim3(FAST_BS), s->stream,
+                           m->dev, m->mst, sfd, K, st, s->d_err);
             else
                 launch_pdl(k_stream_fast<S, A, NQ, false>, dim3((N + FAST_BS - 1) / FAST_BS, 1), dim3(FAST_BS),
                            s->stream, m->dev, m->mst, scd, sfd, K, st, dep);
@@ -765,6 +770,12 @@ cudaError_t launch_step(alelb_solver *s, const StateDev<S> &st0, KinParams<A> &K
             mlp_propose(s, sfd);
             break;
         case KT_MOMENTS:
+            if constexpr (std::is_same<S, float>::value) {
+                if (fused) {
+                    launch_pdl(k_moments_pending, dim3(2 * s->n_sm), dim3(256), s->stream, K, st, N, s->d_err);
+                    break;
+                }
+            }
             launch_pdl(k_moments<S, A>, dim3((N + 255) / 256), dim3(256), s->stream, K, st, N, s->d_err);
             break;
         case KT_DERIV1:

@@ -1145,6 +1145,74 @@ __global__ void __launch_bounds__(256) k_moments(KinParams<A> K, StateDev<S> st,
     if (a < N) moments_node(K, st, N, err, a);
 }
 
+// The FP32 form's propagation and moments in one pass on large meshes, one
+// thread per node: the settled pairs stay in shared memory (a thread reads back
+// its own) and the node's moments follow, exactly as k_moments computes them,
+// unless a population went to the exact path or its wall condition: then the
+// node is listed and k_moments_pending takes it.  Spares k_moments the second
+// reading of the pairs.
+template <int T>
+__global__ void __launch_bounds__(T) k_stream_fast_moments(MeshDev M, MapStatic MS, MapScalarsF sf, KinParams<float> K,
+                                                           StateDev<float> st, int *err)
+{
+    wait_prior_grid();
+    __shared__ float fs[NQ][T], gs[NQ][T];
+    const int tx = threadIdx.x, a = blockIdx.x * T + tx;
+    int code[NQ];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) code[i] = 0;
+    if (a < M.N) {
+        int c[NQ];
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) c[i] = st.cache[i * M.N + a];
+        const float bd = M.bdist[a];
+        const float4 Xf = M.Xf[a];
+        FastMap F = fast_map(MS, sf, a, Xf);
+        if (K.flags & (FLAG_LITERAL_VG | FLAG_EXACT_CHAR)) F.ok = false;
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+            float fo = 0.f, go = 0.f;
+            code[i] = stream_fast_pop(M, K, st, a, i, F, Xf, bd, c[i], fo, go);
+            fs[i][tx] = fo;
+            gs[i][tx] = go;
+        }
+    }
+    int any = 0;
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) any |= code[i];
+    const unsigned pm = __ballot_sync(0xffffffffu, any != 0);
+    if (pm) {
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) append_pop(st, a, M.N, i, code[i]);
+        const unsigned lane = threadIdx.x & 31u;
+        const int leader = __ffs(pm) - 1;
+        unsigned base = 0;
+        if ((int)lane == leader) base = atomicAdd(st.wcount + SEG_PENDING, (unsigned)__popc(pm));
+        base = __shfl_sync(0xffffffffu, base, leader);
+        if (any) st.work[(size_t)SEG_PENDING * M.N + base + __popc(pm & ((1u << lane) - 1u))] = a;
+    }
+    if (a < M.N && !any) {
+        float f[NQ], g[NQ];
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+            f[i] = fs[i][tx];
+            g[i] = gs[i][tx];
+        }
+        moments_store(K, st, err, a, f, g);
+    }
+}
+
+// The moments of the nodes listed as pending, dealt out over the grid; the
+// list itself is emptied by k_collide, once every reader is done.
+static __global__ void __launch_bounds__(256) k_moments_pending(KinParams<float> K, StateDev<float> st, int N, int *err)
+{
+    wait_prior_grid();
+    const unsigned total = st.wcount[SEG_PENDING], first = blockIdx.x * blockDim.x + threadIdx.x;
+    for (unsigned w = first; w < total; w += gridDim.x * blockDim.x)
+        moments_node(K, st, N, err, st.work[(size_t)SEG_PENDING * N + w]);
+    if (first <= (unsigned)NQ) st.wcount[first] = 0u; // the exact path's list has been consumed
+}
+
 // FP32 owner-element derivative d K / d X (rows of the FP32 inverse
 // Jacobian: grad xi = (j11, j12), grad eta = (j21, j22)).
 __constant__ float c_dNxif[6][6];
@@ -1379,6 +1447,7 @@ __global__ void __launch_bounds__(128) k_collide(MeshDev M, MapStatic MS, MapSca
 {
     wait_prior_grid();
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a == 0 && st.wcount) st.wcount[SEG_PENDING] = 0u;
     if (a < M.N) collide_at<S, A>(M, MS, sc, sf, K, st, err, a);
 }
 
