@@ -120,9 +120,8 @@ __device__ __forceinline__ double f2d_bits(float v)
     return __hiloint2double((int)hi, (int)(m >= 0x00800000u ? b << 29 : 0u));
 }
 
-// v 2^k by the exponent field (|k| <= 2), off the FP64 pipe: exact for zero
-// and numbers well inside the range, others are returned unscaled (they occur
-// as shape-function factors below 1e-300 only).
+// v 2^k by the exponent field (|k| <= 3), off the FP64 pipe: exact for zero,
+// infinities and numbers from 2^-1015 to 2^1016; others are returned unscaled.
 __device__ __forceinline__ double scale2_bits(double v, int k)
 {
     const int hi = __double2hiint(v);

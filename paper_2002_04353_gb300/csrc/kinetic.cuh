@@ -235,19 +235,21 @@ __device__ __forceinline__ bool collide_node(const KinParams<A> &K, A f[NQ], A g
 //   diagonal  T^2 M0 / 4 + T (+-Mx +-My) / 4 + (W0 (Nxx + Nyy) +- 2 Mxy) / 8
 // (W0 = 1 - T; psi's (1 - 3T)/T terms cancel the 1/T of the quadratic ones).
 // It is linear in (M0, M, N), so g* - g^eq is the same form of the moments'
-// difference.  About 240 operations per node for moments and collision, four
-// of them divisions, against about 620 with the general forms written out
-// (150,400 nodes: 31 + 131 us before).
+// difference.  Powers of two go by the exponent field (scale2_bits: the same
+// bits), and the two relaxation rates share one division.  About 215
+// operations per node for moments and collision, three of them divisions,
+// against about 620 with the general forms written out (150,400 nodes: 31 +
+// 131 us before).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void gform_psi64(double T, double M0, double Mx, double My, double Nxx, double Mxy,
                                             double Nyy, double G[NQ])
 {
     const double W0 = 1.0 - T, p = W0 * M0, S = Nxx + Nyy, u = 1.0 + T;
-    const double tp = 0.5 * T * p, h = 0.5 * W0, lx = h * Mx, ly = h * My;
-    const double ax = tp + 0.25 * (u * Nxx - W0 * Nyy), ay = tp + 0.25 * (u * Nyy - W0 * Nxx);
-    const double q = 0.25 * T, d = q * T * M0 + 0.125 * W0 * S, e = 0.25 * Mxy;
+    const double tp = scale2_bits(T * p, -1), h = scale2_bits(W0, -1), lx = h * Mx, ly = h * My;
+    const double ax = tp + scale2_bits(u * Nxx - W0 * Nyy, -2), ay = tp + scale2_bits(u * Nyy - W0 * Nxx, -2);
+    const double q = scale2_bits(T, -2), d = q * T * M0 + scale2_bits(W0, -3) * S, e = scale2_bits(Mxy, -2);
     const double dx = q * Mx, dy = q * My, dp = d + e, dm_ = d - e, sp = dx + dy, sm = dx - dy;
-    G[0] = W0 * p - 0.5 * u * S;
+    G[0] = W0 * p - scale2_bits(u, -1) * S;
     G[1] = ax + lx;
     G[2] = ay + ly;
     G[3] = ax - lx;
@@ -273,7 +275,7 @@ __device__ __forceinline__ void fields64(const KinParams<double> &K, const doubl
     wy = jy * r;
     ux = wx + K.Ux;
     uy = wy + K.Uy;
-    T = 0.5 * (sg * r - (ux * ux + uy * uy)) * K.iCv;
+    T = scale2_bits(sg * r - (ux * ux + uy * uy), -1) * K.iCv;
 }
 
 // The collision of one node from its streamed populations and its fields
@@ -286,27 +288,30 @@ __device__ __forceinline__ void collide_node64(const KinParams<double> &K, doubl
     const double s57 = f[5] + f[7], s68 = f[6] + f[8], sd = s57 + s68;
     const double Pxx = (f[1] + f[3]) + sd, Pyy = (f[2] + f[4]) + sd, Pxy = s57 - s68;
     const double M0 = g[0] + ((g[1] + g[2]) + (g[3] + g[4])) + ((g[5] + g[6]) + (g[7] + g[8])); // 2 rho E
-    const double p = rho * T, rx = rho * wx, b = 2.0 * p;
+    const double p = rho * T, rx = rho * wx, b = scale2_bits(p, 1);
     const double dPxx = (Pxx - p) - rx * wx, dPxy = Pxy - rx * wy, dPyy = (Pyy - p) - rho * wy * wy;
-    const double om = 1.0 / (mrt + 0.5), om1 = 1.0 / (mrt * K.iPr + 0.5);
+    const double d0 = mrt + 0.5, d1 = mrt * K.iPr + 0.5, di = 1.0 / (d0 * d1), om = d1 * di, om1 = d0 * di;
     // f toward rho Phi Phi
     const double xT = wx * wx + T, yT = wy * wy + T;
-    const double xz = rho * (1.0 - xT), xp = rho * (0.5 * (xT + wx)), xm = rho * (0.5 * (xT - wx));
-    const double yz = 1.0 - yT, yp = 0.5 * (yT + wy), ym = 0.5 * (yT - wy);
+    // (xp, xm, yp, ym: twice the factors of the moving velocities)
+    const double xz = rho * (1.0 - xT), xp = rho * (xT + wx), xm = rho * (xT - wx);
+    const double yz = 1.0 - yT, yp = yT + wy, ym = yT - wy;
+    const double yzh = scale2_bits(yz, -1), xzh = scale2_bits(xz, -1), xpq = scale2_bits(xp, -2), xmq = scale2_bits(xm, -2);
+    const double hx = scale2_bits(Xx, -1), hy = scale2_bits(Xy, -1);
     f[0] += om * (xz * yz - f[0]);
-    f[1] += om * (xp * yz - f[1]) + 0.5 * Xx; // phi_i = A_ia X_a: +-X/2 on the axis velocities
-    f[2] += om * (xz * yp - f[2]) + 0.5 * Xy;
-    f[3] += om * (xm * yz - f[3]) - 0.5 * Xx;
-    f[4] += om * (xz * ym - f[4]) - 0.5 * Xy;
-    f[5] += om * (xp * yp - f[5]);
-    f[6] += om * (xm * yp - f[6]);
-    f[7] += om * (xm * ym - f[7]);
-    f[8] += om * (xp * ym - f[8]);
+    f[1] += om * (xp * yzh - f[1]) + hx; // phi_i = A_ia X_a: +-X/2 on the axis velocities
+    f[2] += om * (xzh * yp - f[2]) + hy;
+    f[3] += om * (xm * yzh - f[3]) - hx;
+    f[4] += om * (xzh * ym - f[4]) - hy;
+    f[5] += om * (xpq * yp - f[5]);
+    f[6] += om * (xmq * yp - f[6]);
+    f[7] += om * (xmq * ym - f[7]);
+    f[8] += om * (xpq * ym - f[8]);
     // g toward g^eq at omega1, with (omega1 - omega)(g* - g^eq)
     const double Mb = M0 + b, x2 = ux * ux, y2 = uy * uy, xy = ux * uy;
     const double Mx = ux * Mb, My = uy * Mb;
     double Nxx = M0 * x2 + b * (T + 2.0 * x2), Nyy = M0 * y2 + b * (T + 2.0 * y2), Mxy = (Mb + b) * xy;
-    const double c = 2.0 * (om1 - om);
+    const double c = scale2_bits(om1 - om, 1);
     const double Dx = c * (ux * dPxx + uy * dPxy), Dy = c * (ux * dPxy + uy * dPyy);
     double G[NQ];
     if (shift) {
@@ -321,7 +326,7 @@ __device__ __forceinline__ void collide_node64(const KinParams<double> &K, doubl
         for (int i = 0; i < NQ; ++i) g[i] += om1 * (G[i] - g[i]) + D[i];
     } else {
         gform_psi64(T, M0, Mx, My, Nxx, Mxy, Nyy, G);
-        const double h = 0.5 * (1.0 - T), q = 0.25 * T;
+        const double h = scale2_bits(1.0 - T, -1), q = scale2_bits(T, -2);
         const double lx = h * Dx, ly = h * Dy, sp = q * (Dx + Dy), sm = q * (Dx - Dy);
         g[0] += om1 * (G[0] - g[0]);
         g[1] += om1 * (G[1] - g[1]) + lx;
