@@ -308,12 +308,12 @@ __global__ void k_fill_uniform(StateDev<S> st, int N, const double *consts, doub
 //
 // Import was bound by the FP64 pipe (two lanes per SM and clock): about 70
 // operations per node and population set for the differences, sums, moments
-// and conversions (495 us for both sets at 2.0M nodes, 70 of HBM traffic; 192
+// and conversions (495 us for both sets at 2.0M nodes, 70 of HBM traffic; 149
 // us now, in one pass on the device exchange).  The
 // deviation forms now split and sum in 64-bit fixed point: a value below 2 is
 // q 2^-58, rounded once (3.5e-18 at most, half an FP64 ulp of 0.03), its
 // differences and sums are exact integers, and a difference is rounded to FP32
-// once.  About 30 FP64 operations are left per node for both sets.  A node with
+// once.  About 20 FP64 operations are left per node for both sets.  A node with
 // a value outside that range (or not finite) takes the FP64 arithmetic.
 // ---------------------------------------------------------------------------
 constexpr int FIX_BITS = 58;
@@ -361,13 +361,14 @@ __device__ __forceinline__ float fix_to_float(long long q)
     return q < 0 ? -f : f;
 }
 
-// A stored value as FP64: by its bits (f2d_bits) where they are a normal
-// number, spared the FP64 pipe's conversion.
+// A stored deviation as FP64 by its bits, off the FP64 pipe: exact but for
+// subnormal ones, which become zero (they vanish in the reference's rounding).
 __device__ __forceinline__ double widen(double v) { return v; }
 __device__ __forceinline__ double widen(float v)
 {
-    const unsigned m = __float_as_uint(v) & 0x7fffffffu;
-    return m - 0x00800000u < 0x7f000000u ? f2d_bits(v) : (double)v;
+    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+    const unsigned up = m >= 0x7f800000u ? 0x70000000u : m >= 0x00800000u ? 0x38000000u : 0u; // infinite, NaN; normal
+    return __hiloint2double((int)(up ? (b & 0x80000000u) | ((m >> 3) + up) : 0u), (int)(up ? b << 29 : 0u));
 }
 
 // A block's copies of the 18 reference populations and their fixed-point
@@ -453,21 +454,34 @@ __device__ __forceinline__ NodeSums import_half(const RefTable &R, const V v[NQ]
     return r;
 }
 
-// rho and u = sum (c_i + U) f_i / rho from the f set's sums.
+// rho and u = sum (c_i + U) f_i / rho from the f set's sums.  The fields of the
+// deviation forms are rounded to FP32 afterwards, so one reciprocal serves
+// them.
+template <class S>
 __device__ __forceinline__ void import_velocity(const NodeSums &F, double Ux, double Uy, double &ux, double &uy)
 {
-    ux = F.x / F.s + Ux;
-    uy = F.y / F.s + Uy;
+    if constexpr (std::is_same<S, double>::value) {
+        ux = F.x / F.s + Ux;
+        uy = F.y / F.s + Uy;
+    } else {
+        const double r = 1.0 / F.s;
+        ux = F.x * r + Ux;
+        uy = F.y * r + Uy;
+    }
 }
 template <class S>
 __device__ __forceinline__ void import_fields(const StateDev<S> &st, int a, double rho, double ux, double uy, double sg,
-                                              double Cv)
+                                              double Cv, double iCv)
 {
-    const double E = sg / (2 * rho);
     st.rho[a] = (fld_t<S>)rho;
     st.ux[a] = (fld_t<S>)ux;
     st.uy[a] = (fld_t<S>)uy;
-    st.T[a] = (fld_t<S>)((E - 0.5 * (ux * ux + uy * uy)) / Cv);
+    if constexpr (std::is_same<S, double>::value) {
+        const double E = sg / (2 * rho);
+        st.T[a] = (E - 0.5 * (ux * ux + uy * uy)) / Cv;
+    } else {
+        st.T[a] = (fld_t<S>)((0.5 * (sg * (1.0 / rho) - (ux * ux + uy * uy))) * iCv);
+    }
 }
 
 // Host exchange, one population set per launch so that each half's kernel
@@ -479,7 +493,7 @@ __device__ __forceinline__ void import_fields(const StateDev<S> &st, int a, doub
 template <class S, class V>
 __global__ void __launch_bounds__(256) k_import(StateDev<S> st, int N, const double *__restrict__ consts,
                                                 const V *__restrict__ plane, const double *__restrict__ fields,
-                                                double Cv, double Ux, double Uy, const int *__restrict__ n2o,
+                                                double Cv, double iCv, double Ux, double Uy, const int *__restrict__ n2o,
                                                 double *tmp, int part)
 {
     __shared__ RefTable R;
@@ -497,7 +511,7 @@ __global__ void __launch_bounds__(256) k_import(StateDev<S> st, int N, const dou
     if (part == 0) {
         if (!fields) {
             double ux, uy;
-            import_velocity(n, Ux, Uy, ux, uy);
+            import_velocity<S>(n, Ux, Uy, ux, uy);
             tmp[a] = n.s;
             tmp[N + a] = ux;
             tmp[2 * N + a] = uy;
@@ -508,7 +522,7 @@ __global__ void __launch_bounds__(256) k_import(StateDev<S> st, int N, const dou
         st.uy[a] = (fld_t<S>)fields[2 * N + o];
         st.T[a] = (fld_t<S>)fields[3 * N + o];
     } else {
-        import_fields(st, a, tmp[a], tmp[N + a], tmp[2 * N + a], n.s, Cv);
+        import_fields(st, a, tmp[a], tmp[N + a], tmp[2 * N + a], n.s, Cv, iCv);
     }
 }
 
@@ -516,7 +530,7 @@ __global__ void __launch_bounds__(256) k_import(StateDev<S> st, int N, const dou
 template <class S>
 __global__ void __launch_bounds__(256) k_import_dev(StateDev<S> st, int N, const double *__restrict__ consts,
                                                     const double *__restrict__ f, const double *__restrict__ g,
-                                                    double Cv, double Ux, double Uy, const int *__restrict__ n2o)
+                                                    double Cv, double iCv, double Ux, double Uy, const int *__restrict__ n2o)
 {
     __shared__ RefTable R;
     R.load(consts);
@@ -534,13 +548,13 @@ __global__ void __launch_bounds__(256) k_import_dev(StateDev<S> st, int N, const
 #pragma unroll
     for (int i = 0; i < NQ; ++i) fg_put(st.post, i, a, N, df[i], dg[i]);
     double ux, uy;
-    import_velocity(F, Ux, Uy, ux, uy);
-    import_fields(st, a, F.s, ux, uy, G.s, Cv);
+    import_velocity<S>(F, Ux, Uy, ux, uy);
+    import_fields(st, a, F.s, ux, uy, G.s, Cv, iCv);
 }
 
 // The sets as full FP64 populations into the caller's planes, one set per grid
-// row and one plane at a time (2.0M nodes: 150 us with the loads of nine or
-// eighteen planes together ahead of their scattered stores).
+// row and one plane at a time, the widening by bits (2.0M nodes: 125 us; 150
+// with the loads of nine or eighteen planes ahead of their scattered stores).
 template <class S>
 __global__ void __launch_bounds__(256) k_export_dev(StateDev<S> st, int N, const double *consts, double *f, double *g,
                                                     const int *n2o)
@@ -563,10 +577,10 @@ __global__ void k_fields_dev(StateDev<S> st, int N, double *rho, double *ux, dou
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= N) return;
     const int o = n2o[a];
-    if (rho) rho[o] = widen(st.rho[a]);
-    if (ux) ux[o] = widen(st.ux[a]);
-    if (uy) uy[o] = widen(st.uy[a]);
-    if (T) T[o] = widen(st.T[a]);
+    if (rho) rho[o] = (double)st.rho[a];
+    if (ux) ux[o] = (double)st.ux[a];
+    if (uy) uy[o] = (double)st.uy[a];
+    if (T) T[o] = (double)st.T[a];
 }
 
 // Export: part 0 the f deviations, part 1 the g deviations.
@@ -1068,7 +1082,7 @@ cudaError_t alelb::import_enqueue(alelb_solver *s, const double *f, const double
     const dim3 grid((N + 255) / 256), block(256);
     with_state(s, [&](auto &sx, auto &) {
         k_import<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, (const double *)s->d_scratch,
-                                                (const double *)(have ? dfields : nullptr), s->Cv, s->U[0], s->U[1],
+                                                (const double *)(have ? dfields : nullptr), s->Cv, 1.0 / s->Cv, s->U[0], s->U[1],
                                                 s->mesh->d_n2o, dfields, 0);
     });
     st = cudaGetLastError();
@@ -1076,7 +1090,7 @@ cudaError_t alelb::import_enqueue(alelb_solver *s, const double *f, const double
     if (st == cudaSuccess)
         with_state(s, [&](auto &sx, auto &) {
             k_import<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, (const double *)(s->d_scratch + (size_t)9 * N),
-                                                    (const double *)(have ? dfields : nullptr), s->Cv, s->U[0], s->U[1],
+                                                    (const double *)(have ? dfields : nullptr), s->Cv, 1.0 / s->Cv, s->U[0], s->U[1],
                                                     s->mesh->d_n2o, dfields, 1);
         });
     if (st == cudaSuccess) st = cudaGetLastError();
@@ -1122,12 +1136,12 @@ cudaError_t alelb::import_stored_enqueue(alelb_solver *s, const float *f, const 
     if (st == cudaSuccess) st = cudaEventRecord(s->ev_copy[1], s->copy_stream);
     if (st != cudaSuccess) return st;
     const dim3 grid((N + 255) / 256), block(256);
-    k_import<<<grid, block, 0, s->stream>>>(s->sf, N, s->d_consts, (const float *)pf, (const double *)nullptr, s->Cv,
+    k_import<<<grid, block, 0, s->stream>>>(s->sf, N, s->d_consts, (const float *)pf, (const double *)nullptr, s->Cv, 1.0 / s->Cv,
                                             s->U[0], s->U[1], s->mesh->d_n2o, tmp, 0);
     st = cudaGetLastError();
     if (st == cudaSuccess) st = cudaStreamWaitEvent(s->stream, s->ev_copy[1], 0);
     if (st == cudaSuccess) {
-        k_import<<<grid, block, 0, s->stream>>>(s->sf, N, s->d_consts, (const float *)pg, (const double *)nullptr, s->Cv,
+        k_import<<<grid, block, 0, s->stream>>>(s->sf, N, s->d_consts, (const float *)pg, (const double *)nullptr, s->Cv, 1.0 / s->Cv,
                                                 s->U[0], s->U[1], s->mesh->d_n2o, tmp, 1);
         st = cudaGetLastError();
     }
@@ -1199,7 +1213,7 @@ extern "C" alelb_status alelb_set_pops_dev(alelb_solver *s, const double *f, con
     const int N = s->mesh->T.N;
     const dim3 grid((N + 255) / 256), block(256);
     with_state(s, [&](auto &sx, auto &) {
-        k_import_dev<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, f, g, s->Cv, s->U[0], s->U[1], s->mesh->d_n2o);
+        k_import_dev<<<grid, block, 0, s->stream>>>(sx, N, s->d_consts, f, g, s->Cv, 1.0 / s->Cv, s->U[0], s->U[1], s->mesh->d_n2o);
     });
     cudaError_t st = cudaGetLastError();
     if (st == cudaSuccess) st = cudaStreamSynchronize(s->stream);
