@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(256) k_export_dev(StateDev<S> st, int N, const
                                                     const int *n2o)
 {
     const int a = blockIdx.x * blockDim.x + threadIdx.x, part = blockIdx.y;
-    if (a >= N) return;
+    if (a >= N || (part == 0 && f == g)) return; // one buffer for both keeps the g set
     const int o = n2o[a];
     double *plane = part ? g : f;
 #pragma unroll 1

@@ -546,9 +546,9 @@ __global__ void __launch_bounds__(128) k_stream(MeshDev M, MapStatic MS, MapScal
 
 // ---------------------------------------------------------------------------
 // The propagation, split by path so that the rare exact work does not
-// stall the warps of the common case (FP64 form, 150,400-node plunge: 103 +
-// 43 + 31 us for the three kernels against 1,194 us in one pass with every
-// population walked in FP64; 9,216-node box 20 + 28 + 12 against 268 us):
+// stall the warps of the common case (FP64 form, 150,400-node plunge: 80 +
+// 38 + 17 us for the three kernels against 1,194 us in one pass with every
+// population walked in FP64; 9,216-node box 16 + 24 + 5 against 268 us):
 //   k_stream_fast  per population: FP32 map; a population whose
 //                  previous-step element is verified (fast_decide) is
 //                  interpolated and stored, one certified missing by the

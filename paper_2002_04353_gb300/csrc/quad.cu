@@ -7,7 +7,7 @@
 // Eq. Propagation and the element gradients (quad.cuh).  Every form first
 // tries the previous-step element under a certified FP32 test
 // (quad_fast_decide); the other populations take the exact FP64 path.  The
-// FP64 form at 150,400 nodes (plunge): 225 + 67 us for the two passes against
+// FP64 form at 150,400 nodes (plunge): 147 + 41 us for the two passes against
 // 3,881 us with every population walked and Newton in FP64.
 #include <cuda_runtime.h>
 
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(128) kq_stream(QuadDev M, MapStatic MS, MapSca
 // map is a translation (no map, plunge).  The lanes are brought together after
 // the certified test and after Newton (__syncwarp): left apart, the own and the
 // other elements' lanes interpolated one after the other (150,400 nodes: 60 us
-// against 33 in FP32, 408 against 175 in FP64).  FP32 is held to 32 registers,
+// against 33 in FP32, 408 against 175 in FP64 at the time).  FP32 is held to 32 registers,
 // 16 blocks an SM (35 us at 40).
 template <class S, class A, int G, bool TR>
 __global__ void __launch_bounds__(128, std::is_same<S, double>::value ? 1 : 16) kq_fast(QuadDev M, MapStatic MS, MapScalars scd, MapScalarsF sfd,
