@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("blended", [True, False])
 def test_moments_along_with_the_propagation(blended):
-    c = I.pitch_case(ni=451, nj=168, Ma=0.3, blended=blended)
+    c = I.pitch_case(ni=450, nj=168, Ma=0.3, blended=blended)
     assert c.mesh.n_nodes >= 300000 and c.mesh.n_nodes % 128
     flow = dataclasses.replace(c.flow, flags=alelb.FLAG_OFFWALL_VG)
     m = alelb.Mesh(c.mesh, c.motion)
