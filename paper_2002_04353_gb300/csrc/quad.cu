@@ -33,8 +33,8 @@ __device__ __forceinline__ bool quad_fast_pop(const QuadDev &M, const FastMap &F
     float cw[8];
     float xi, eta;
     bool in = quad_fast_decide(M, F, Xf, a, i, c, e, cw);
-    __syncwarp(lanes);
-    if (in) in = quad_newton_t<float>(cw, 1e-5f, 1e-4f, xi, eta);
+    const unsigned newton = __ballot_sync(lanes, in); // the lanes that iterate together
+    if (in) in = quad_newton_t<float>(cw, 1e-5f, 1e-4f, xi, eta, newton);
     __syncwarp(lanes);
     if (!in) return false;
     A Nw[9];
@@ -63,7 +63,7 @@ __device__ __forceinline__ bool quad_fast_pop64(const QuadDev &M, const FastMap 
     float cw[8];
     double px, py, xi, eta, f, g;
     bool in = quad_fast_decide(M, F, Xf, a, i, c, e, cw);
-    __syncwarp(lanes);
+    const unsigned newton = __ballot_sync(lanes, in);
     if (in) {
         if (TR) {
             const double2 cw = D.c[i];
@@ -72,7 +72,7 @@ __device__ __forceinline__ bool quad_fast_pop64(const QuadDev &M, const FastMap 
         } else {
             departure64<TR>(n, i, X, px, py);
         }
-        in = quad_local64(M, e, 0, 0, px, py, xi, eta);
+        in = quad_local64(M, e, 0, 0, px, py, xi, eta, newton);
     }
     __syncwarp(lanes);
     if (!in) return false;

@@ -49,20 +49,22 @@ ALELB_HD __forceinline__ void quad_bilinear(const double w[8], double xi, double
 // element choice never depends on it (exact signs decide), only the
 // interpolation weights.
 constexpr int QUAD_NEWTON_ITERS = 8;
-// Whether any lane of the warp's running ones still iterates: the lanes leave
-// the loop together (a lane that has converged keeps its values meanwhile), so
-// that the interpolation after it runs once per warp, not once per iteration
-// count (kq_fast at 150,400 nodes: 56 us with lanes leaving one by one).
-ALELB_HD __forceinline__ bool lanes_go(bool go)
+// Whether any lane of `lanes` still iterates: those lanes leave the loop
+// together (a lane that has converged keeps its values meanwhile), so that the
+// interpolation after it runs once per warp, not once per iteration count
+// (kq_fast at 150,400 nodes: 56 us with lanes leaving one by one).  Every lane
+// of the mask has to come here, which only the caller can know: it votes for
+// the mask before its lanes part (quad_fast_pop).  lanes = 0: the lane is on its
+// own, as on the exact path, where the lanes of a warp are at different entries.
+ALELB_HD __forceinline__ bool lanes_go(unsigned lanes, bool go)
 {
 #ifdef __CUDA_ARCH__
-    return __any_sync(__activemask(), go);
-#else
-    return go;
+    if (lanes) return __any_sync(lanes, go);
 #endif
+    return go;
 }
 template <class A>
-ALELB_HD __forceinline__ bool quad_newton_t(const A c[8], A done, A tol, A &xi, A &eta)
+ALELB_HD __forceinline__ bool quad_newton_t(const A c[8], A done, A tol, A &xi, A &eta, unsigned lanes = 0)
 {
     A a = A(0), b = A(0), da = A(0), db = A(0);
     bool go = true;
@@ -86,7 +88,7 @@ ALELB_HD __forceinline__ bool quad_newton_t(const A c[8], A done, A tol, A &xi, 
             b -= db;
             go = !(fabs(da) + fabs(db) < done);
         }
-        if (!lanes_go(go)) break;
+        if (!lanes_go(lanes, go)) break;
     }
     xi = a;
     eta = b;
@@ -520,7 +522,7 @@ __device__ __forceinline__ float d2f_bits(double v)
 // of every operation is pinned, so the result is the same in every kernel.
 // false: the corrections did not settle (the last one above 1e-9).
 __device__ __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, int sy, double px, double py,
-                                             double &xi, double &eta)
+                                             double &xi, double &eta, unsigned lanes = 0)
 {
     double2 b0 = M.ebd[4 * e];
     const double2 b1 = M.ebd[4 * e + 1], b2 = M.ebd[4 * e + 2], b3 = M.ebd[4 * e + 3];
@@ -553,7 +555,7 @@ __device__ __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, in
             v = __fadd_rn(v, dv);
             go = !(fabsf(du) + fabsf(dv) < 1e-4f); // the next step would be below the FP32 rounding
         }
-        if (!lanes_go(go)) break;
+        if (!lanes_go(lanes, go)) break;
     }
     inverse();
     xi = f2d_bits(u);
