@@ -77,7 +77,7 @@ alelb_status check_sticky(alelb_solver *s)
 
 namespace {
 
-template <class S> void put_state(DevBuf &b, StateDev<S> &s, int N, int mkind, cudaError_t &st)
+template <class S> void put_state(DevBuf &b, StateDev<S> &s, int N, int mkind, int flags, cudaError_t &st)
 {
     using P = pop_t<S>;
     using F = fld_t<S>;
@@ -97,7 +97,10 @@ template <class S> void put_state(DevBuf &b, StateDev<S> &s, int N, int mkind, c
     s.work = b.alloc<int>((size_t)(SEG_PENDING + 1) * N, st);
     s.wcount = b.alloc<unsigned>(SEG_PENDING + 1, st);
     if (st == cudaSuccess) st = cudaMemset(s.wcount, 0, (SEG_PENDING + 1) * sizeof(unsigned));
-    s.met = std::is_same<S, double>::value && !uniform_metric(mkind) ? b.alloc<double2>((size_t)2 * N, st) : nullptr;
+    // the propagation leaves the metrics of the arrival time only where it evaluates the map of that time, in two
+    // passes; under the other options there is no such array, and the derivative passes evaluate the map
+    const bool left = !uniform_metric(mkind) && !(flags & (FLAG_LITERAL_VG | FLAG_EXACT_CHAR | FLAG_MIDPOINT));
+    s.met = std::is_same<S, double>::value && left ? b.alloc<double2>((size_t)2 * N, st) : nullptr;
     s.wmask = b.alloc<unsigned>(N, st);
     if (st == cudaSuccess) st = cudaMemset(s.wmask, 0, (size_t)N * sizeof(unsigned));
 }
@@ -660,12 +663,8 @@ cudaEvent_t get_event(alelb_solver *s)
 
 
 template <class S, class A>
-cudaError_t launch_step(alelb_solver *s, const StateDev<S> &st0, KinParams<A> &K, const MapScalars &sc_in)
+cudaError_t launch_step(alelb_solver *s, StateDev<S> &st, KinParams<A> &K, const MapScalars &sc_in)
 {
-    StateDev<S> st = st0;
-    // the propagation leaves the metrics only where it evaluates the map of
-    // the arrival time
-    if (s->flags & (ALELB_FLAG_LITERAL_VG | ALELB_FLAG_EXACT_CHAR | ALELB_FLAG_MIDPOINT)) st.met = nullptr;
     alelb_mesh *m = s->mesh;
     const MapScalars sc = solver_map(s, sc_in);
     const int N = m->T.N;
@@ -895,7 +894,7 @@ extern "C" alelb_status alelb_lb_init(alelb_mesh *m, const alelb_params *p, alel
             cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && nsm > 0)
             s->n_sm = nsm;
     }
-    with_state(s, [&](auto &sx, auto &) { put_state(s->buf, sx, N, m->T.mkind, st); });
+    with_state(s, [&](auto &sx, auto &) { put_state(s->buf, sx, N, m->T.mkind, s->flags, st); });
     s->d_consts = s->buf.alloc<double>(4 * NQ, st);
     s->d_scratch = s->buf.alloc<double>((size_t)22 * N, st);
     s->d_err = s->buf.alloc<int>(1, st);
