@@ -311,16 +311,27 @@ __global__ void k_fill_uniform(StateDev<S> st, int N, const double *consts, doub
 //
 // Import was bound by the FP64 pipe (two lanes per SM and clock): about 70
 // operations per node and population set for the differences, sums, moments
-// and conversions (495 us for both sets at 2.0M nodes, 70 of HBM traffic; 149
-// us now, in one pass on the device exchange).  The
-// deviation forms now split and sum in 64-bit fixed point: a value below 2 is
-// q 2^-58, rounded once (3.5e-18 at most, half an FP64 ulp of 0.03), its
-// differences and sums are exact integers, and a difference is rounded to FP32
-// once.  About 20 FP64 operations are left per node for both sets.  A node with
-// a value outside that range (or not finite) takes the FP64 arithmetic.
+// and conversions (495 us for both sets at 2.0M nodes, 70 of HBM traffic; 134
+// us now, in one pass on the device exchange).  The deviation forms now split
+// and sum in 64-bit fixed point.  Its unit goes with the references, so that the
+// result does not depend on the density's scale: the largest of them lies in
+// [2^57, 2^58) units.  A value is rounded to a unit once (exact from 2^-6 of
+// that range on), differences and sums are exact integers, and a difference is
+// rounded to FP32 once.  About 20 FP64 operations are left per node for both
+// sets.  The FP64 arithmetic is taken by a node with a value beyond the range (or
+// not finite), by all nodes if no unit fits the references, and where the unit
+// would show: by a node that has values or references so small that they may not
+// be whole numbers of units (below 2^52), and either a difference below 2^34
+// units or a sum below SUM_MIN.
 // ---------------------------------------------------------------------------
 constexpr int FIX_BITS = 58;
-constexpr double FIX_UNIT = 1.0 / (double)(1ll << FIX_BITS);
+constexpr int FIX_MIN = -60, FIX_MAX = 36; // the shift's range: the FP32 scale below stays a normal number
+// From this sum on the nine roundings to a unit stay below the rounding of the
+// sum in FP64 (2^-53 of it).
+constexpr long long SUM_MIN = 1ll << 54;
+// Two roundings to a unit are 2^-34 of the difference (DIFF_MIN = 2^34 units, here
+// in units of 2^32).
+constexpr int DIFF_HI = 4;
 
 // m 2^s, rounded to nearest (m < 2^53, s <= 35 and m 2^s < 2^60).
 __device__ __forceinline__ long long fix_shift(unsigned long long m, int s, bool neg)
@@ -333,34 +344,38 @@ __device__ __forceinline__ long long fix_shift(unsigned long long m, int s, bool
     }
     return neg ? -(long long)m : (long long)m;
 }
-// v in units of 2^-FIX_BITS; false when v is not finite or |v| >= 2 (an FP32
-// deviation: 1).
-__device__ __forceinline__ bool to_fix(double v, long long &q)
+// v in units of 2^-(FIX_BITS + sh); false when v is not finite or beyond 2^59
+// units (an FP32 deviation: 2^58).  rough is set when v may not be a whole
+// number of units.
+__device__ __forceinline__ bool to_fix(double v, int sh, long long &q, bool &rough)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const int e = (int)(b >> 52) & 0x7ff;
+    const int e = (int)(b >> 52) & 0x7ff, s = min(max(e, 1) - (1075 - FIX_BITS) + sh, 6);
     const unsigned long long m = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
-    q = fix_shift(m, min(max(e, 1) - (1075 - FIX_BITS), 6), (long long)b < 0);
-    return e <= 1023;
+    rough |= s < 0;
+    q = fix_shift(m, s, (long long)b < 0);
+    return e <= 1023 - sh;
 }
-__device__ __forceinline__ bool to_fix(float v, long long &q)
+__device__ __forceinline__ bool to_fix(float v, int sh, long long &q, bool &rough)
 {
     const unsigned b = __float_as_uint(v);
-    const int e = (int)(b >> 23) & 0xff;
+    const int e = (int)(b >> 23) & 0xff, s = min(max(e, 1) - (150 - FIX_BITS) + sh, 35);
     const unsigned long long m = (b & 0x7fffffu) | (e ? 1u << 23 : 0u);
-    q = fix_shift(m, min(max(e, 1) - (150 - FIX_BITS), 35), (int)b < 0);
-    return e <= 126; // |v| < 1: nine sums of a deviation and its reference stay below 2^63
+    rough |= s < 0;
+    q = fix_shift(m, s, (int)b < 0);
+    // nine sums of a deviation and its reference stay below 2^63; 255: not finite
+    return e <= min(126 - sh, 254);
 }
-// q 2^-FIX_BITS rounded to FP32: the upper 32 bits of |q| with the rest as a
-// sticky bit, through the 32-bit conversion.
-__device__ __forceinline__ float fix_to_float(long long q)
+// q 2^-(FIX_BITS + sh) rounded to FP32: the upper 32 bits of |q| with the rest
+// as a sticky bit, through the 32-bit conversion.
+__device__ __forceinline__ float fix_to_float(long long q, int sh)
 {
     const unsigned long long m = (unsigned long long)(q < 0 ? -q : q);
     if (m == 0) return 0.f;
     const int n = __clzll((long long)m);
     const unsigned long long y = m << n;
     const unsigned h = (unsigned)(y >> 32) | ((unsigned)y ? 1u : 0u);
-    const float f = __uint2float_rn(h) * __uint_as_float((unsigned)(127 + 32 - FIX_BITS - n) << 23);
+    const float f = __uint2float_rn(h) * __uint_as_float((unsigned)(127 + 32 - FIX_BITS - n - sh) << 23);
     return q < 0 ? -f : f;
 }
 
@@ -374,21 +389,36 @@ __device__ __forceinline__ double widen(float v)
     return __hiloint2double((int)(up ? (b & 0x80000000u) | ((m >> 3) + up) : 0u), (int)(up ? b << 29 : 0u));
 }
 
-// A block's copies of the 18 reference populations and their fixed-point
-// values.
+// A block's copies of the 18 reference populations, their fixed-point values
+// and the unit.
 struct RefTable {
-    double c[2 * NQ];
+    double c[2 * NQ], unit;
     long long q[2 * NQ];
-    int ok;
+    int sh, ok, rough; // rough: some may not be a whole number of units
     __device__ void load(const double *consts)
     {
-        bool in = true;
-        if (threadIdx.x < 2 * NQ) {
-            c[threadIdx.x] = consts[threadIdx.x];
-            in = to_fix(consts[threadIdx.x], q[threadIdx.x]);
+        if (threadIdx.x < 32) {
+            const int k = threadIdx.x;
+            const double v = k < 2 * NQ ? consts[k] : 0.0;
+            const unsigned top = __reduce_max_sync(0xffffffffu, (unsigned)(__double_as_longlong(v) >> 52) & 0x7ffu);
+            const int s = 1022 - (int)top;
+            const bool reach = s >= FIX_MIN && s <= FIX_MAX;
+            long long fix;
+            bool rest = false;
+            const bool in = to_fix(v, reach ? s : 0, fix, rest);
+            if (k < 2 * NQ) {
+                c[k] = v;
+                q[k] = fix;
+            }
+            const bool r = __any_sync(0xffffffffu, rest && k < 2 * NQ);
+            const bool all = __all_sync(0xffffffffu, in);
+            if (k == 0) {
+                sh = reach ? s : 0;
+                unit = __hiloint2double((1023 - FIX_BITS - (reach ? s : 0)) << 20, 0);
+                ok = reach && all;
+                rough = r;
+            }
         }
-        const int all = __syncthreads_and(in);
-        if (threadIdx.x == 0) ok = all;
         __syncthreads();
     }
 };
@@ -420,14 +450,17 @@ __device__ __forceinline__ NodeSums import_half(const RefTable &R, const V v[NQ]
     } else {
         long long q[NQ];
         bool in = R.ok != 0;
+        bool rough = R.rough != 0, small = false;
 #pragma unroll
-        for (int i = 0; i < NQ; ++i) in &= to_fix(v[i], q[i]);
+        for (int i = 0; i < NQ; ++i) in &= to_fix(v[i], R.sh, q[i], rough);
         if (in) {
 #pragma unroll
             for (int i = 0; i < NQ; ++i) {
                 const long long c = R.q[part * NQ + i];
                 if constexpr (std::is_same<V, double>::value) {
-                    d[i] = fix_to_float(q[i] - c);
+                    const long long dq = q[i] - c;
+                    d[i] = fix_to_float(dq, R.sh);
+                    small |= (unsigned)((int)(dq >> 32) + DIFF_HI) < 2u * DIFF_HI;
                 } else {
                     d[i] = v[i];
                     q[i] += c;
@@ -435,10 +468,12 @@ __device__ __forceinline__ NodeSums import_half(const RefTable &R, const V v[NQ]
             }
             long long s, x, y;
             lattice_sums(q, s, x, y);
-            r.s = (double)s * FIX_UNIT;
-            r.x = (double)x * FIX_UNIT;
-            r.y = (double)y * FIX_UNIT;
-        } else {
+            in = !rough || (!small && s >= SUM_MIN);
+            r.s = (double)s * R.unit;
+            r.x = (double)x * R.unit;
+            r.y = (double)y * R.unit;
+        }
+        if (!in) {
             double w[NQ];
 #pragma unroll
             for (int i = 0; i < NQ; ++i) {
