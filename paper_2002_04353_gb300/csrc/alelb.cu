@@ -379,16 +379,6 @@ __device__ __forceinline__ float fix_to_float(long long q, int sh)
     return q < 0 ? -f : f;
 }
 
-// A stored deviation as FP64 by its bits, off the FP64 pipe: exact but for
-// subnormal ones, which become zero (they vanish in the reference's rounding).
-__device__ __forceinline__ double widen(double v) { return v; }
-__device__ __forceinline__ double widen(float v)
-{
-    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
-    const unsigned up = m >= 0x7f800000u ? 0x70000000u : m >= 0x00800000u ? 0x38000000u : 0u; // infinite, NaN; normal
-    return __hiloint2double((int)(up ? (b & 0x80000000u) | ((m >> 3) + up) : 0u), (int)(up ? b << 29 : 0u));
-}
-
 // A block's copies of the 18 reference populations, their fixed-point values
 // and the unit.
 struct RefTable {
@@ -591,8 +581,9 @@ __global__ void __launch_bounds__(256) k_import_dev(StateDev<S> st, int N, const
 }
 
 // The sets as full FP64 populations into the caller's planes, one set per grid
-// row and one plane at a time, the widening by bits (2.0M nodes: 125 us; 150
-// with the loads of nine or eighteen planes ahead of their scattered stores).
+// row and one plane at a time: bound by the scattered stores (2.0M nodes: 146 us
+// in FP32, 139 in FP16; one launch per set took 149 and 144, and the loads of
+// nine or eighteen planes ahead of their stores gained nothing).
 template <class S>
 __global__ void __launch_bounds__(256) k_export_dev(StateDev<S> st, int N, const double *consts, double *f, double *g,
                                                     const int *n2o)
@@ -605,7 +596,7 @@ __global__ void __launch_bounds__(256) k_export_dev(StateDev<S> st, int N, const
     for (int i = 0; i < NQ; ++i) {
         fld_t<S> x, y;
         fg_get(st.post, i, a, N, x, y);
-        plane[(size_t)i * N + o] = widen(part ? y : x) + consts[part * NQ + i];
+        plane[(size_t)i * N + o] = (double)(part ? y : x) + consts[part * NQ + i];
     }
 }
 template <class S>
