@@ -121,7 +121,7 @@ struct TrainSmem {
     float X[TS][8], B[TS][4];
     float W1[MLP_H * MLP_IN], b1[MLP_H], b2[MLP_H], b3[LO];
     int SL[TS], NR[TS];
-    float L[TRAIN_THREADS / 32];
+    double L[TRAIN_THREADS / 32];
 };
 
 __device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
@@ -201,7 +201,7 @@ k_mlp_fwd_bwd(const __half *__restrict__ Wh, const float *__restrict__ feat,
     // dW3 rows 4 ty .., columns 4 tx .., and rows 32 .. 34 by column; dW1 row
     // tid % 64, three columns; the biases by column
     float g2[2][4][4] = {}, g3[4][4] = {}, g3r[2] = {}, g1[3] = {}, gb1 = 0.f, gb2 = 0.f, gb3 = 0.f;
-    float loss = 0.f;
+    double loss = 0.0; // of the warp's samples, in lane 0
     const float inv_cnt = 1.0f / (float)cnt;
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         if (tile != (int)blockIdx.x) {
@@ -308,8 +308,13 @@ k_mlp_fwd_bwd(const __half *__restrict__ Wh, const float *__restrict__ feat,
             for (int c = 0; c < MLP_K / 4; ++c) o[r + 4 * c] = dv[c];
             const float gd = r < 3 ? og - S.B[s][r] : 0.f;
             o[MLP_K + r] = in && r < 3 ? w_bary * 2.0f * gd / 3.0f * inv_cnt : 0.f;
-            if (in) loss += w_bary * (gd * gd) / 3.0f;
-            if (in && r == 0) loss += -(osl - m - lz);
+            // the tile's loss: FP32 over the warp's eight samples, FP64 from
+            // there on, as a block's tiles grow with the number of samples
+            float ls = in ? w_bary * (gd * gd) / 3.0f : 0.f;
+            if (in && r == 0) ls += -(osl - m - lz);
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) ls += __shfl_xor_sync(0xffffffffu, ls, off);
+            if ((tid & 31) == 0) loss += (double)ls;
         }
         __syncthreads();
         // dW3 (and its bias): outer products over the samples
@@ -431,12 +436,11 @@ k_mlp_fwd_bwd(const __half *__restrict__ Wh, const float *__restrict__ feat,
         P[MLP_OFF_B2 + tid] = gb2;
     }
     if (tid >= 64 && tid < 64 + MLP_OUT) P[MLP_OFF_B3 + tid - 64] = gb3;
-    for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
     if ((tid & 31) == 0) S.L[tid >> 5] = loss;
     __syncthreads();
     if (tid == 0) {
         double l = 0.0;
-        for (int w = 0; w < TRAIN_THREADS / 32; ++w) l += (double)S.L[w];
+        for (int w = 0; w < TRAIN_THREADS / 32; ++w) l += S.L[w];
         lpart[blockIdx.x] = l;
     }
 }
