@@ -296,9 +296,12 @@ __device__ __forceinline__ unsigned quad_slow_pop(const QuadDev &M, const MapSta
             set_err(err, ERR_LOCATE);
         quad_interp64(M, st.post, N, i, L.e, xi, eta, fi, gi);
     } else {
-        pr.load(L.e, L.sx, L.sy); // the walk may end in the neighbour across an edge
-        const float c[8] = {pr.x0 + chx, pr.y0 + chy, pr.x1 + chx, pr.y1 + chy,
-                            pr.x2 + chx, pr.y2 + chy, pr.x3 + chx, pr.y3 + chy};
+        const double2 X = M.X[a];
+        const Node64 n = node64<false>(MS, scd, a, X, false);
+        double px, py;
+        departure64<false>(n, i, X, px, py);
+        float c[8];
+        quad_corners32(M, L.e, L.sx, L.sy, px, py, c);
         float xi, eta;
         if (!quad_newton_t<float>(c, 1e-5f, 1e-4f, xi, eta)) set_err(err, ERR_LOCATE);
         A Nw[9];

@@ -501,6 +501,25 @@ ALELB_HD __forceinline__ bool quad_local(const QuadDev &M, int e, int sx, int sy
     return quad_newton_t<A>(c, A(1e-5), A(1e-4), xi, eta); // FP32: converged near 1e-7
 }
 
+// The corners of element e (frame shift sx, sy) relative to the FP64 point p,
+// as FP32 numbers: the shift is taken from p in FP64, then the leading and the
+// trailing parts (corner and point split in two FP32 numbers each) are
+// subtracted, the former exactly, so that one rounding remains (quad_local's
+// FP32 corners in eight FP64 subtractions and conversions less).
+ALELB_HD __forceinline__ void quad_corners32(const QuadDev &M, int e, int sx, int sy, double px, double py, float c[8])
+{
+    if (sx) px = px - sx * M.Lx;
+    if (sy) py = py - sy * M.Ly;
+    const float hx = (float)px, hy = (float)py;
+    const float lx = (float)(px - (double)hx), ly = (float)(py - (double)hy);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4 v = M.evf[4 * e + k];
+        c[2 * k] = (v.x - hx) + (v.z - lx);
+        c[2 * k + 1] = (v.y - hy) + (v.w - ly);
+    }
+}
+
 // FP64 <-> FP32 by their bits, for values whose rounding does not matter
 // (the FP64 pipe runs conversions at its own low rate): truncation toward
 // zero, below the normal range to zero, above it to the largest float.
