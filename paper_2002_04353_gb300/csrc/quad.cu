@@ -341,10 +341,13 @@ __global__ void __launch_bounds__(128) kq_stream(QuadDev M, MapStatic MS, MapSca
 // map is a translation (no map, plunge).  The lanes are brought together after
 // the certified test and after Newton (__syncwarp): left apart, the own and the
 // other elements' lanes interpolated one after the other (150,400 nodes: 60 us
-// against 33 in FP32, 408 against 175 in FP64 at the time).  FP32 is held to 32 registers,
-// 16 blocks an SM (35 us at 40).
+// against 33 in FP32).  The FP32 and 16-bit forms are held to 32 registers, 16
+// blocks an SM, on a translation (33 us; 35 at 40 registers), and to 40, 12 blocks,
+// on the other maps, which spill at 32 (150,400 nodes pitching: 37.1 us, 38.3 at
+// 32 registers and 39.1 at 48; blended 37.8, 39.3, 40.1; 600,996 nodes 129 at 32
+// and 40, 141 at 48).
 template <class S, class A, int G, bool TR>
-__global__ void __launch_bounds__(128, std::is_same<S, double>::value ? 1 : 16) kq_fast(QuadDev M, MapStatic MS, MapScalars scd, MapScalarsF sfd,
+__global__ void __launch_bounds__(128, std::is_same<S, double>::value ? 1 : TR ? 16 : 12) kq_fast(QuadDev M, MapStatic MS, MapScalars scd, MapScalarsF sfd,
                                                KinParams<A> K, StateDev<S> st, unsigned long long *stats,
                                                const __grid_constant__ DepTab D)
 {
