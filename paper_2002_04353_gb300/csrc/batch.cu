@@ -90,6 +90,21 @@ template <class S, class A> struct SharedCase {
     }
 };
 
+// The FP64 form's plain pass (plain_pass).
+__global__ void __launch_bounds__(256) kb_stream(const CaseDev<double, double> *__restrict__ cases,
+                                                 const int *__restrict__ off, int B,
+                                                 const MapScalars *__restrict__ sc, int count)
+{
+    wait_prior_grid();
+    __shared__ SharedCase<double, double> sh;
+    const int c = tile_case(off, B, blockIdx.x);
+    sh.load(cases, sc, nullptr, c);
+    __syncthreads();
+    const CaseDev<double, double> &C = sh.C();
+    const int a = (blockIdx.x - __ldg(off + c)) * blockDim.x + threadIdx.x;
+    if (a < C.M.N) stream_plain_node(C.M, C.MS, sh.SC(), sh.SC(), C.K, C.st, C.err, count ? C.stats : nullptr, a);
+}
+
 // G directions per thread (grid y: 9 / G groups), chosen by the tuner:
 // one map evaluation per thread, fewer and longer load chains as G grows.
 template <class S, class A, int G>
@@ -776,12 +791,28 @@ void drop_graphs(alelb_batch *b)
     b->graphs.clear();
 }
 
+// FP64 cases that all run the literal velocities keep the plain pass, as the
+// single solver does: no FP32 certificate covers their departure points, so the
+// first of the two passes would only list every population (4 cases of 100k
+// nodes: 3,127 us a step against 3,520; of 20k nodes 780 against 834).
+bool plain_pass(const alelb_batch *b)
+{
+    if (b->prec != ALELB_PREC_FP64) return false;
+    for (const alelb_solver *s : b->cs)
+        if (!(s->flags & ALELB_FLAG_LITERAL_VG)) return false;
+    return true;
+}
+
 // Phase kernels of one step, in order.
-int step_sequence(int seq[KT_N])
+int step_sequence(const alelb_batch *b, int seq[KT_N])
 {
     int n = 0;
-    seq[n++] = KT_FAST;
-    seq[n++] = KT_SLOW;
+    if (plain_pass(b)) {
+        seq[n++] = KT_STREAM;
+    } else {
+        seq[n++] = KT_FAST;
+        seq[n++] = KT_SLOW;
+    }
     seq[n++] = KT_MOMENTS;
     seq[n++] = KT_DERIV1;
     seq[n++] = KT_COLLIDE;
@@ -843,6 +874,10 @@ void launch_phase(alelb_batch *b, const Part &P, int kt, int bs, int grid, int k
     const int B = P.B;
     const bool fast = b->prec == ALELB_PREC_FP32_DEV;
     switch (kt) {
+    case KT_STREAM:
+        if constexpr (std::is_same<S, double>::value)
+            launch_after(P.pdl, kb_stream, dim3(tiles), dim3(bs), P.stream, cases, off, B, sc, count);
+        break;
     case KT_FAST:
         // fast_g: directions per thread, plus FAST_FUSED for the propagation
         // fused with the moments
@@ -948,7 +983,7 @@ template <class S, class A> int persistent_grid_t(int bs, int n_sm)
 void enqueue_step(alelb_batch *b, int k)
 {
     int seq[KT_N];
-    const int ns = step_sequence(seq);
+    const int ns = step_sequence(b, seq);
     for (int q = 0; q < ns; ++q) {
         const int kt = seq[q];
         cudaEvent_t ea = nullptr, eb = nullptr;
@@ -974,7 +1009,7 @@ void enqueue_step(alelb_batch *b, int k)
 cudaError_t enqueue_groups(alelb_batch *b, int k)
 {
     int seq[KT_N];
-    const int ns = step_sequence(seq);
+    const int ns = step_sequence(b, seq);
     const int lead = std::min(b->pipe ? (b->pipe == 2 ? 2 : 1) : 0, ns);
     cudaError_t st = cudaSuccess;
     for (int g = 0; g < b->groups && st == cudaSuccess; ++g) {
@@ -1467,7 +1502,7 @@ extern "C" alelb_status alelb_batch_tune(alelb_batch *b, int32_t reps, int32_t c
     if (st == cudaSuccess) st = cudaEventCreate(&e1);
     if (st != cudaSuccess) return bfail(b, st, "batch_tune");
     int seq[KT_N];
-    const int ns = step_sequence(seq);
+    const int ns = step_sequence(b, seq);
     const auto clear = [b]() {
         if (b->prec == ALELB_PREC_FP32_DEV)
             kb_clear_work<float, float>
@@ -1700,7 +1735,7 @@ extern "C" alelb_status alelb_batch_step_host(alelb_batch *b, const float *const
     cudaError_t st = stage_scalars(b, 0, 1); // the map scalars of time t_c + 1
     if (st == cudaSuccess) st = cudaEventRecord(b->gev_fork, b->stream);
     int seq[KT_N];
-    const int ns = step_sequence(seq);
+    const int ns = step_sequence(b, seq);
     for (int g = 0; g < P && st == cudaSuccess; ++g) {
         Part G = part(g);
         // the group's uploads, after the previous group's
