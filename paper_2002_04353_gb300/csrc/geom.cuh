@@ -113,11 +113,48 @@ ALELB_HD __forceinline__ void set_err(int *err, int bit)
 
 // A float as a double by its bits (the FP64 pipe runs conversions at its own
 // low rate): exact for 0 and normal numbers; a subnormal one is not kept.
-__device__ __forceinline__ double f2d_bits(float v)
+ALELB_HD __forceinline__ double f2d_bits(float v)
 {
+#ifndef __CUDA_ARCH__
+    return v == 0.0f || std::fabs(v) >= 1.17549435e-38f ? (double)v : 0.0;
+#else
     const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
     const unsigned hi = m >= 0x00800000u ? (b & 0x80000000u) | ((m >> 3) + 0x38000000u) : 0u;
     return __hiloint2double((int)hi, (int)(m >= 0x00800000u ? b << 29 : 0u));
+#endif
+}
+// FP32 operations that round once each, never fused (as dm, da, ds, dfma).
+ALELB_HD __forceinline__ float fm(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+ALELB_HD __forceinline__ float fa(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fadd_rn(a, b);
+#else
+    return a + b;
+#endif
+}
+ALELB_HD __forceinline__ float ffma(float a, float b, float c)
+{
+#ifdef __CUDA_ARCH__
+    return __fmaf_rn(a, b, c);
+#else
+    return std::fma(a, b, c);
+#endif
+}
+ALELB_HD __forceinline__ float frcp(float a)
+{
+#ifdef __CUDA_ARCH__
+    return __frcp_rn(a);
+#else
+    return 1.0f / a;
+#endif
 }
 
 // v 2^k by the exponent field (|k| <= 3), off the FP64 pipe: exact for zero,

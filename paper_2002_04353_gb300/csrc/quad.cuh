@@ -145,7 +145,7 @@ struct QuadDev {
     const float *bdist;    // [N] lower bound of the distance to the nearest boundary edge
     const float4 *ownJf;   // [N] owner element's J^{-1} at the node, FP32
     const double2 *ownJd;  // [2N] the same in FP64 (grad xi, grad eta)
-    const double2 *ebd;    // [4E] bilinear map: x = b0 + b1 xi + b2 eta + b3 xi eta
+    const double2 *ebd;    // [5E] bilinear map (QuadTables)
     const float4 *cone;    // [N] boundary node: outgoing, incoming boundary edge (as MeshDev's)
     const uint8_t *conek;  // [N]
     const uint8_t *vzero;  // [N] 1: mesh velocity exactly zero at all times
@@ -523,55 +523,79 @@ ALELB_HD __forceinline__ void quad_corners32(const QuadDev &M, int e, int sx, in
 // FP64 <-> FP32 by their bits, for values whose rounding does not matter
 // (the FP64 pipe runs conversions at its own low rate): truncation toward
 // zero, below the normal range to zero, above it to the largest float.
-__device__ __forceinline__ float d2f_bits(double v)
+ALELB_HD __forceinline__ float d2f_bits(double v)
 {
-    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v), m = hi & 0x7fffffffu;
+#ifdef __CUDA_ARCH__
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+#else
+    unsigned long long w;
+    std::memcpy(&w, &v, 8);
+    const unsigned hi = (unsigned)(w >> 32), lo = (unsigned)w;
+#endif
+    const unsigned m = hi & 0x7fffffffu;
     unsigned b = ((m - 0x38000000u) << 3) | (lo >> 29);
     if (m < 0x38100000u) b = 0u;
     if (m >= 0x47f00000u) b = 0x7f7fffffu;
-    return __uint_as_float(b | (hi & 0x80000000u));
+    b |= hi & 0x80000000u;
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(b);
+#else
+    float f;
+    std::memcpy(&f, &b, 4);
+    return f;
+#endif
 }
 
 // Local coordinates of p in element e for the FP64 form: Newton in FP32 on
-// the bilinear map x = b0 + b1 xi + b2 eta + b3 xi eta, then two corrections
-// with the residual in FP64 and the FP32 inverse Jacobian.  A correction
-// leaves about 2^-20 of the error it finds (2^-20 after the FP32 part), so
-// two of them end at the rounding of the residual; each costs 13 operations
-// of the FP64 pipe, against about 60 for a Newton step in FP64.  The rounding
-// of every operation is pinned, so the result is the same in every kernel.
-// false: the corrections did not settle (the last one above 1e-9).
-__device__ __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, int sy, double px, double py,
-                                             double &xi, double &eta, unsigned lanes = 0)
+// the bilinear map x = w0 + c + b1 xi + b2 eta + b3 xi eta, then corrections
+// with the residual in FP64 and the FP32 inverse Jacobian.  A correction leaves
+// a part k of the error it finds: the FP32 rounding of the Jacobian, 2^-20 in
+// cells near a parallelogram of moderate aspect, more by the aspect ratio in
+// thin cells oblique to the axes (1e-3 at 1e4).  The last two corrections give
+// it, k = last / before, so what the last one leaves is last^2 / before: after
+// two, more are made while that is above 2^-54 (none on the O-meshes and boxes;
+// 2^-52: the rounding of the coordinates).  The residual is formed from the
+// point relative to a corner, exact nearby, by fused operations; a correction
+// costs 9 operations of the FP64 pipe, against about 60 for a Newton step in
+// FP64.  The error against extended precision is that of Newton's method in FP64
+// on the corners relative to p: in the quadratic mean over the cells 4.1e-17
+// (Newton 6.4e-17) on a jittered box, 5.5e-17 (7.4e-17) on the 150k O-mesh,
+// 8.6e-17 (9.1e-17) on one of 64 x 20 cells; at most 1.7e-16 (2.6e-16), 2.0e-15
+// (1.1e-15), 3.9e-15 (3.0e-15).  The rounding of every operation is pinned, so
+// the result is the same in every kernel.  false: the corrections did not settle (the last one above 1e-9).
+constexpr int QUAD_CORRECTIONS = 4;
+ALELB_HD __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, int sy, double px, double py,
+                                           double &xi, double &eta, unsigned lanes = 0)
 {
-    double2 b0 = M.ebd[4 * e];
-    const double2 b1 = M.ebd[4 * e + 1], b2 = M.ebd[4 * e + 2], b3 = M.ebd[4 * e + 3];
-    if (sx) b0.x = da(b0.x, sx * M.Lx);
-    if (sy) b0.y = da(b0.y, sy * M.Ly);
-    const double dx = ds(px, b0.x), dy = ds(py, b0.y);
+    double2 w0 = M.ebd[5 * e];
+    const double2 b1 = M.ebd[5 * e + 1], b2 = M.ebd[5 * e + 2], b3 = M.ebd[5 * e + 3], c = M.ebd[5 * e + 4];
+    if (sx) w0.x = da(w0.x, sx * M.Lx);
+    if (sy) w0.y = da(w0.y, sy * M.Ly);
+    const double dx = ds(ds(px, w0.x), c.x), dy = ds(ds(py, w0.y), c.y);
     const float fx = d2f_bits(dx), fy = d2f_bits(dy);
     const float b1x = d2f_bits(b1.x), b1y = d2f_bits(b1.y), b2x = d2f_bits(b2.x), b2y = d2f_bits(b2.y),
                 b3x = d2f_bits(b3.x), b3y = d2f_bits(b3.y);
     float u = 0.f, v = 0.f, i11 = 0.f, i12 = 0.f, i21 = 0.f, i22 = 0.f;
     const auto inverse = [&]() { // J^{-1} at (u, v)
-        const float j11 = __fmaf_rn(b3x, v, b1x), j12 = __fmaf_rn(b3x, u, b2x);
-        const float j21 = __fmaf_rn(b3y, v, b1y), j22 = __fmaf_rn(b3y, u, b2y);
-        const float inv = __frcp_rn(__fmaf_rn(j11, j22, -__fmul_rn(j12, j21)));
-        i11 = __fmul_rn(j22, inv);
-        i12 = -__fmul_rn(j12, inv);
-        i21 = -__fmul_rn(j21, inv);
-        i22 = __fmul_rn(j11, inv);
+        const float j11 = ffma(b3x, v, b1x), j12 = ffma(b3x, u, b2x);
+        const float j21 = ffma(b3y, v, b1y), j22 = ffma(b3y, u, b2y);
+        const float inv = frcp(ffma(j11, j22, -fm(j12, j21)));
+        i11 = fm(j22, inv);
+        i12 = -fm(j12, inv);
+        i21 = -fm(j21, inv);
+        i22 = fm(j11, inv);
     };
     bool go = true;
 #pragma unroll 1
     for (int it = 0; it < QUAD_NEWTON_ITERS; ++it) {
         if (go) {
             inverse();
-            const float uv = __fmul_rn(u, v);
-            const float rx = __fsub_rn(fx, __fmaf_rn(b3x, uv, __fmaf_rn(b2x, v, __fmul_rn(b1x, u))));
-            const float ry = __fsub_rn(fy, __fmaf_rn(b3y, uv, __fmaf_rn(b2y, v, __fmul_rn(b1y, u))));
-            const float du = __fmaf_rn(i11, rx, __fmul_rn(i12, ry)), dv = __fmaf_rn(i21, rx, __fmul_rn(i22, ry));
-            u = __fadd_rn(u, du);
-            v = __fadd_rn(v, dv);
+            const float uv = fm(u, v);
+            const float rx = fa(fx, -ffma(b3x, uv, ffma(b2x, v, fm(b1x, u))));
+            const float ry = fa(fy, -ffma(b3y, uv, ffma(b2y, v, fm(b1y, u))));
+            const float du = ffma(i11, rx, fm(i12, ry)), dv = ffma(i21, rx, fm(i22, ry));
+            u = fa(u, du);
+            v = fa(v, dv);
             go = !(fabsf(du) + fabsf(dv) < 1e-4f); // the next step would be below the FP32 rounding
         }
         if (!lanes_go(lanes, go)) break;
@@ -579,18 +603,23 @@ __device__ __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, in
     inverse();
     xi = f2d_bits(u);
     eta = f2d_bits(v);
-    float du = 0.f, dv = 0.f;
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
+    float last = 0.f, left = 0.f; // the last correction, what it leaves
+    const auto correct = [&]() {
         const double q = dm(xi, eta);
-        const float rx = d2f_bits(ds(dx, dfma(b3.x, q, dfma(b2.x, eta, dm(b1.x, xi)))));
-        const float ry = d2f_bits(ds(dy, dfma(b3.y, q, dfma(b2.y, eta, dm(b1.y, xi)))));
-        du = __fmaf_rn(i11, rx, __fmul_rn(i12, ry));
-        dv = __fmaf_rn(i21, rx, __fmul_rn(i22, ry));
+        const float rx = d2f_bits(dfma(-b3.x, q, dfma(-b2.x, eta, dfma(-b1.x, xi, dx))));
+        const float ry = d2f_bits(dfma(-b3.y, q, dfma(-b2.y, eta, dfma(-b1.y, xi, dy))));
+        const float du = ffma(i11, rx, fm(i12, ry)), dv = ffma(i21, rx, fm(i22, ry));
+        const float before = last;
         xi = da(xi, f2d_bits(du));
         eta = da(eta, f2d_bits(dv));
-    }
-    return fabsf(du) <= 1e-9f && fabsf(dv) <= 1e-9f;
+        last = fabsf(du) + fabsf(dv); // (a sum, so that one that is not a number stays so)
+        left = fm(last, last) - fm(5.5511151231257827e-17f, before); // 2^-54
+    };
+    correct();
+    correct();
+#pragma unroll 1
+    for (int it = 2; it < QUAD_CORRECTIONS && !(left <= 0.f || last <= 2.220446049250313e-16f); ++it) correct();
+    return last <= 1e-9f;
 }
 
 // The pair (f_i, g_i) of the FP64 form interpolated at (xi, eta) of element
@@ -663,7 +692,7 @@ __device__ __forceinline__ void quad_grad3_linear(const QuadDev &M, int2 el, con
     const int e = el.x, l = el.y;
     const int ix = quad_ix(l) - 1, iy = quad_iy(l) - 1;
     const double xi = ix < 0 ? -1.0 : ix ? 1.0 : 0.0, eta = iy < 0 ? -1.0 : iy ? 1.0 : 0.0;
-    const double2 b1 = M.ebd[4 * e + 1], b2 = M.ebd[4 * e + 2], b3 = M.ebd[4 * e + 3];
+    const double2 b1 = M.ebd[5 * e + 1], b2 = M.ebd[5 * e + 2], b3 = M.ebd[5 * e + 3];
     const double jxx = b1.x + b3.x * eta, jxe = b2.x + b3.x * xi, jyx = b1.y + b3.y * eta, jye = b2.y + b3.y * xi;
     const double inv = 1.0 / (jxx * jye - jyx * jxe);
     int nb[4];

@@ -33,11 +33,55 @@ struct QuadTables {
     // bilinear map's coefficients of each element, and the nodes whose mesh
     // velocity is zero at all times
     std::vector<double2> ownJd; // [2N]
-    std::vector<double2> ebd;   // [4E] b0, b1, b2, b3: x = b0 + b1 xi + b2 eta + b3 xi eta
+    std::vector<double2> ebd;   // [5E] w0, b1, b2, b3, c: x = w0 + c + b1 xi + b2 eta + b3 xi eta, w0 the first corner
     std::vector<uint8_t> vzero; // [N]
     std::vector<float4> cone;   // [N] exterior cones (build_cones)
     std::vector<uint8_t> conek; // [N]
 };
+
+// Coefficients of the bilinear map of the corners v (QuadTables::ebd).  Sums of
+// corner differences, rounded once: the rounding errors of the differences and
+// their sums are summed beside them.
+inline void quad_map_coefficients(const double2 v[4], double2 out[5])
+{
+    struct Sum {
+        double s = 0.0, err = 0.0;
+        void add(double x)
+        {
+            const double t = s + x, b = t - s;
+            err += (s - (t - b)) + (x - b);
+            s = t;
+        }
+        void diff(double a, double b) // + a - b
+        {
+            const double d = a - b, c = d - a;
+            err += (a - (d - c)) - (b + c);
+            add(d);
+        }
+        double quarter() const { return 0.25 * (s + err); }
+    };
+    const auto coef = [](double a, double b, double c, double d, double o[5]) {
+        Sum b1, b2, b3, m;
+        b1.diff(b, a);
+        b1.diff(c, d);
+        b2.diff(d, a);
+        b2.diff(c, b);
+        b3.diff(c, d);
+        b3.diff(a, b);
+        m.diff(b, a);
+        m.diff(d, a);
+        m.diff(c, a);
+        o[0] = a;
+        o[1] = b1.quarter();
+        o[2] = b2.quarter();
+        o[3] = b3.quarter();
+        o[4] = m.quarter();
+    };
+    double x[5], y[5];
+    coef(v[0].x, v[1].x, v[2].x, v[3].x, x);
+    coef(v[0].y, v[1].y, v[2].y, v[3].y, y);
+    for (int k = 0; k < 5; ++k) out[k] = make_double2(x[k], y[k]);
+}
 
 // Local coordinates of p in the quadrilateral with corners w (x, y pairs),
 // by the Newton iteration the kernels use (centre start, QUAD_NEWTON_ITERS
@@ -377,22 +421,8 @@ inline alelb_status build_quad_tables(const alelb_mesh_desc *d, HostTables &T, Q
         Q.ownJd[2 * a] = make_double2(J[3] / det, -J[1] / det);
         Q.ownJd[2 * a + 1] = make_double2(-J[2] / det, J[0] / det);
     }
-    Q.ebd.resize((size_t)4 * E);
-    for (int e = 0; e < E; ++e) {
-        const double2 *v = Q.ev.data() + (size_t)4 * e;
-        // differences of the corners (exact for nearby coordinates), then halves and sums
-        auto coef = [](double a, double b, double c, double d, double o[4]) {
-            const double u = b - a, w = c - d; // along the lower and the upper edge
-            o[0] = 0.25 * (((a + b) + c) + d);
-            o[1] = 0.25 * (u + w);
-            o[2] = 0.25 * ((d - a) + (c - b));
-            o[3] = 0.25 * (w - u);
-        };
-        double bx[4], by[4];
-        coef(v[0].x, v[1].x, v[2].x, v[3].x, bx);
-        coef(v[0].y, v[1].y, v[2].y, v[3].y, by);
-        for (int k = 0; k < 4; ++k) Q.ebd[(size_t)4 * e + k] = make_double2(bx[k], by[k]);
-    }
+    Q.ebd.resize((size_t)5 * E);
+    for (int e = 0; e < E; ++e) quad_map_coefficients(Q.ev.data() + (size_t)4 * e, Q.ebd.data() + (size_t)5 * e);
     // lower bound of every node's distance to the nearest boundary edge,
     // capped at DCAP (zero on periodic meshes with boundaries: those always
     // walk): a departure segment shorter than it cannot leave the mesh
