@@ -95,7 +95,8 @@ def kernel_bytes(kernel, n_nodes, n_elems, exact_items, pop_bytes=4, fld_bytes=4
                     Q', mu/(rho T) written, FP64 coordinates, fan entries;
                     per element frame, neighbours, edge info, rank,
                     connectivity (92 B)
-    fused           the batched propagation fused with the moments: the
+    fused           the propagation fused with the moments (the batch's fused
+                    form; a single FP32 solver where moments_fused): the
                     propagation also writes Q'_x, Q'_y, mu/(rho T) of its
                     nodes (counted for all N) and lists the pending nodes;
                     the moments kernel reads the list and does the pending
@@ -118,6 +119,15 @@ def kernel_bytes(kernel, n_nodes, n_elems, exact_items, pop_bytes=4, fld_bytes=4
     if kernel == "k_stream":
         return N * (36 * p + 3 * f + 16 + 3 * 8 + 4) + E * 92
     return 0
+
+
+FUSED_NODES = 300000  # FAST_G_NODES of kernels.cuh
+
+
+def moments_fused(fp32, motion_kind, n_nodes):
+    """Whether a single solver's propagation also takes the moments (the rule of the step's launch): FP32 deviations on a map that
+    turns or deforms, from FUSED_NODES nodes on."""
+    return fp32 and motion_kind not in (I.MOTION_NONE, I.MOTION_PLUNGE) and n_nodes >= FUSED_NODES
 
 
 STEP_KERNELS = ("k_stream_fast", "k_stream_slow", "k_moments", "k_deriv1", "k_collide")
@@ -717,7 +727,8 @@ def run_precision(alelb, torch, dev, args, Ma, shift=(0.0, 0.0), flags=0):
         s.close()
         r = {"value": N * K / (ms * 1e-3) / 1e6, "ms_per_step": ms / K, "pop_bytes": pb}
         if prec != alelb.PREC_FP64:
-            step_bytes = sum(kernel_bytes(k, N, E, n_exact, pop_bytes=pb) for k in STEP_KERNELS)
+            fused = moments_fused(prec == alelb.PREC_FP32_DEV, case.motion.kind, N)
+            step_bytes = sum(kernel_bytes(k, N, E, n_exact, pop_bytes=pb, fused=fused) for k in STEP_KERNELS)
             r["algorithmic_bytes_per_step"] = step_bytes
             r["achieved_gbs"] = step_bytes / (ms / K * 1e-3) / 1e9
         if prec == alelb.PREC_FP64:
