@@ -17,7 +17,9 @@ back with CUDA events on the batch's stream.  Beside it: the plain FP64
 single-case form (the comparison the metric names) and the FP32 single
 case on the 150,400-node plunge (L2 flushed before each of its steps), the
 learned proposal on a 2M-node pitching mesh, storage-precision studies,
-force histories, and the FP64 oracle on the host cores.
+force histories, and the FP64 oracle on the host cores.  The headline's
+fields are printed as one JSON line on standard output, everything measured as
+one on standard error before it.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
@@ -1067,8 +1069,7 @@ def run_q2(alelb, torch, dev, args):
     """The paper's own element: the 150,400-node plunging NACA 0012 O-mesh
     of 9-node quadrilaterals (the same rings as the triangle mesh, each cell
     kept whole), FP32-deviation and FP64 forms, L2 flushed before each
-    timed step.  Every population takes the exact path (FP64 departure
-    point, exact walk over quadrilaterals, Newton for Eq. NonLinear_Eq)."""
+    timed step."""
     case = I.plunge_case(elem="q2")
     mesh = alelb.Mesh(case.mesh, case.motion)
     stream = torch.cuda.Stream(device=dev)
@@ -1099,6 +1100,25 @@ def run_q2(alelb, torch, dev, args):
         s.close()
         out[label] = {"value": case.mesh.n_nodes * K / (ms * 1e-3) / 1e6, "unit": UNIT, "ms_per_step": ms / K,
                       "steps": K, "kernels": {k: {"ms_per_launch": v[0] / v[1]} for k, v in kt.items() if v[1]}}
+    return out
+
+
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+            "dtype", "precision", "data", "config", "gpu_launches", "clocks")
+
+
+def headline(line):
+    """The line on standard output: the headline's fields alone, so that a reader who keeps only the end of the output has all of
+    them.  Everything measured goes to standard error before it, as {"detail": ...}."""
+    def pick(key, *names):
+        part = line.get(key)
+        return None if part is None else {n: part[n] for n in names if n in part}
+
+    out = {k: line[k] for k in HEADLINE}
+    out["roofline"] = pick("roofline", "bound", "kernel", "achieved", "peak", "unit", "frac", "peak_source", "traffic")
+    out["step_roofline"] = pick("step_roofline", "method_bytes_per_step", "achieved_gbs", "frac")
+    out["e2e"] = pick("e2e", "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps")
+    out["cpu_baseline"] = pick("cpu_baseline", "value", "unit", "cores", "kind", "cpu_model")
     return out
 
 
@@ -1210,7 +1230,8 @@ def run_ours(args):
             "oracle_timing": oracle_cfg,
             "clocks": bat["clocks"],
         }
-        print(json.dumps(line), flush=True)
+        print(json.dumps({"detail": line}), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
 
