@@ -158,7 +158,9 @@ ALELB_HD __forceinline__ float frcp(float a)
 }
 
 // v 2^k by the exponent field (|k| <= 3), off the FP64 pipe: exact for zero,
-// infinities and numbers from 2^-1015 to 2^1016; others are returned unscaled.
+// infinities and numbers from 2^-1015 to 2^1016; others are returned unscaled,
+// so it serves values that may vanish beside others of middle size (a density at
+// the ends of the range is moved to its middle first, collide_store64).
 __device__ __forceinline__ double scale2_bits(double v, int k)
 {
     const int hi = __double2hiint(v);

@@ -1394,9 +1394,35 @@ __device__ __forceinline__ void collide_store64(const KinParams<double> &K, cons
     double f[NQ], g[NQ];
 #pragma unroll
     for (int i = 0; i < NQ; ++i) fg_get(st.str, i, a, N, f[i], g[i]);
-    const double rho = st.rho[a], T = st.T[a];
-    if (rho > 0.0 && T > 0.0 && !(K.flags & FLAG_COLLIDE_OFF))
+    double rho = st.rho[a];
+    const double T = st.T[a];
+    if (rho > 0.0 && T > 0.0 && !(K.flags & FLAG_COLLIDE_OFF)) {
+        // the powers of two of collide_node64 keep to the middle of the exponent's
+        // range; the collision is linear in the density, so that a node at its ends
+        // is moved there and back
+        const int e = __double2hiint(rho) >> 20;
+        const bool far = (unsigned)(e - 200) > 1640u;
+        if (far) {
+            const double up = e < 1023 ? 0x1p+512 : 0x1p-512;
+            rho *= up;
+            Xx *= up;
+            Xy *= up;
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) {
+                f[i] *= up;
+                g[i] *= up;
+            }
+        }
         collide_node64(K, f, g, rho, st.ux[a], st.uy[a], T, st.mrt[a], Xx, Xy);
+        if (far) {
+            const double down = e < 1023 ? 0x1p-512 : 0x1p+512;
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) {
+                f[i] *= down;
+                g[i] *= down;
+            }
+        }
+    }
 #pragma unroll
     for (int i = 0; i < NQ; ++i) fg_put(st.post, i, a, N, f[i], g[i]);
 }
