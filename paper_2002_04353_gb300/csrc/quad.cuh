@@ -562,7 +562,9 @@ ALELB_HD __forceinline__ float d2f_bits(double v)
 // (Newton 6.4e-17) on a jittered box, 5.5e-17 (7.4e-17) on the 150k O-mesh,
 // 8.6e-17 (9.1e-17) on one of 64 x 20 cells; at most 1.7e-16 (2.6e-16), 2.0e-15
 // (1.1e-15), 3.9e-15 (3.0e-15).  The rounding of every operation is pinned, so
-// the result is the same in every kernel.  false: the corrections did not settle (the last one above 1e-9).
+// the result is the same in every kernel.  false: the corrections did not settle
+// (the last one above 1e-9), or the cell's area is beyond FP32 (an inverse of
+// zero would leave any point settled).
 constexpr int QUAD_CORRECTIONS = 4;
 ALELB_HD __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, int sy, double px, double py,
                                            double &xi, double &eta, unsigned lanes = 0)
@@ -575,11 +577,11 @@ ALELB_HD __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, int 
     const float fx = d2f_bits(dx), fy = d2f_bits(dy);
     const float b1x = d2f_bits(b1.x), b1y = d2f_bits(b1.y), b2x = d2f_bits(b2.x), b2y = d2f_bits(b2.y),
                 b3x = d2f_bits(b3.x), b3y = d2f_bits(b3.y);
-    float u = 0.f, v = 0.f, i11 = 0.f, i12 = 0.f, i21 = 0.f, i22 = 0.f;
+    float u = 0.f, v = 0.f, i11 = 0.f, i12 = 0.f, i21 = 0.f, i22 = 0.f, inv = 0.f;
     const auto inverse = [&]() { // J^{-1} at (u, v)
         const float j11 = ffma(b3x, v, b1x), j12 = ffma(b3x, u, b2x);
         const float j21 = ffma(b3y, v, b1y), j22 = ffma(b3y, u, b2y);
-        const float inv = frcp(ffma(j11, j22, -fm(j12, j21)));
+        inv = frcp(ffma(j11, j22, -fm(j12, j21)));
         i11 = fm(j22, inv);
         i12 = -fm(j12, inv);
         i21 = -fm(j21, inv);
@@ -619,7 +621,7 @@ ALELB_HD __forceinline__ bool quad_local64(const QuadDev &M, int e, int sx, int 
     correct();
 #pragma unroll 1
     for (int it = 2; it < QUAD_CORRECTIONS && !(left <= 0.f || last <= 2.220446049250313e-16f); ++it) correct();
-    return last <= 1e-9f;
+    return last <= 1e-9f && inv != 0.f;
 }
 
 // The pair (f_i, g_i) of the FP64 form interpolated at (xi, eta) of element

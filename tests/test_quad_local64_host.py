@@ -82,3 +82,17 @@ def test_local_coordinates(lib, kind):
     tol = 2.0 ** -52 + 16 * 2.0 ** -53 * (np.abs(inv.reshape(-1, 2, 2)) * ext[:, None, :]).sum(2)
     err = np.abs(np.stack([x, y], 1) - out)
     assert np.all(err <= tol), float((err / tol).max())
+
+
+@pytest.mark.parametrize("size", [1e-25, 1e-19, 1e10, 1e18, 1e20, 1e45])
+def test_cells_beyond_fp32(lib, size):
+    """Where FP32 does not hold a cell's edges or their products the point is left to Newton's method in FP64, or is right."""
+    w = _cells((1, 1.0))[:500] * size
+    p = w.mean(1) + 0.3 * (w[:, 1] - w[:, 0])
+    buf = np.ascontiguousarray(np.concatenate([w.reshape(-1, 8), p], 1))
+    out = np.empty((1, 2))
+    q = np.longdouble
+    x, y, _ = _newton((w / size).astype(q), (p / size).astype(q))
+    for k in range(len(w)):
+        if lib.alelb_hostcheck_local64(1, buf[k].ctypes.data, out.ctypes.data) == 0:
+            assert abs(out[0, 0] - x[k]) < 1e-12 and abs(out[0, 1] - y[k]) < 1e-12
