@@ -254,6 +254,18 @@ __device__ __forceinline__ unsigned quad_stream_pops(const QuadDev &M, const Map
     return walks;
 }
 
+// The departure point of population i of node a; a translation spares the map's
+// chain of operations (150,400 nodes: 1,534 us against 1,560 per 20 FP32 steps,
+// 1,489 against 1,498 per 5 FP64 steps).
+__device__ __forceinline__ void quad_departure64(const MapStatic &MS, const MapScalars &scd, int a, int i, double2 X,
+                                                 double &px, double &py)
+{
+    if (MS.kind == MK_NONE || MS.kind == MK_PLUNGE)
+        departure64<true>(node64<true>(MS, scd, a, X, false), i, X, px, py);
+    else
+        departure64<false>(node64<false>(MS, scd, a, X, false), i, X, px, py);
+}
+
 // Population i of node a on the exact path, its walk on certified FP32
 // predicates: location, interpolation, far-field or wall condition.  Returns
 // the number of walks (0: c^ is exactly zero).  Where no FP32 map is usable the
@@ -288,18 +300,16 @@ __device__ __forceinline__ unsigned quad_slow_pop(const QuadDev &M, const MapSta
         fg_get(st.post, i, L.e == -2 ? a : L.vnode, N, fi, gi);
     } else if constexpr (std::is_same<S, double>::value) {
         const double2 X = M.X[a];
-        const Node64 n = node64<false>(MS, scd, a, X, false);
         double px, py, xi, eta;
-        departure64<false>(n, i, X, px, py);
+        quad_departure64(MS, scd, a, i, X, px, py);
         if (!quad_local64(M, L.e, L.sx, L.sy, px, py, xi, eta) &&
             !quad_local<double>(M, L.e, L.sx, L.sy, px, py, xi, eta))
             set_err(err, ERR_LOCATE);
         quad_interp64(M, st.post, N, i, L.e, xi, eta, fi, gi);
     } else {
         const double2 X = M.X[a];
-        const Node64 n = node64<false>(MS, scd, a, X, false);
         double px, py;
-        departure64<false>(n, i, X, px, py);
+        quad_departure64(MS, scd, a, i, X, px, py);
         float c[8];
         quad_corners32(M, L.e, L.sx, L.sy, px, py, c);
         float xi, eta;
