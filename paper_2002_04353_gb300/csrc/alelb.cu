@@ -838,8 +838,10 @@ template <class A> void fill_kin(alelb_solver *s, KinParams<A> &K)
     K.Cp = (A)s->Cp;
     K.mu = (A)s->mu;
     K.Pr = (A)s->Pr;
-    K.iCv = (A)(1.0 / s->Cv);
-    K.iPr = (A)(1.0 / s->Pr);
+    if constexpr (std::is_same<A, double>::value) {
+        K.iCv = 1.0 / s->Cv;
+        K.iPr = 1.0 / s->Pr;
+    }
     double r = 0, jx = 0, jy = 0, pxx = 0, pxy = 0, pyy = 0, e2 = 0;
     for (int i = 0; i < NQ; ++i) {
         const double fr = s->consts[i];
