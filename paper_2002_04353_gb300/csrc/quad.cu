@@ -7,7 +7,7 @@
 // Eq. Propagation and the element gradients (quad.cuh).  Every form first
 // tries the previous-step element under a certified FP32 test
 // (quad_fast_decide); the other populations take the exact FP64 path.  The
-// FP64 form at 150,400 nodes (plunge): 147 + 41 us for the two passes against
+// FP64 form at 150,400 nodes (plunge): 145 + 40 us for the two passes against
 // 3,881 us with every population walked and Newton in FP64.
 #include <cuda_runtime.h>
 
@@ -422,8 +422,8 @@ __global__ void __launch_bounds__(128, std::is_same<S, double>::value ? 1 : TR ?
 
 // The exact path's walk runs on certified FP32 signs, the wall condition once
 // per wall node for its cone-certified directions, its three gradients with one
-// Jacobian: 31 us against 53 with every listed population walked in FP64 and
-// its wall condition computed per direction (FP32, 150,400 nodes; FP64 form 43
+// Jacobian: 30 us against 53 with every listed population walked in FP64 and
+// its wall condition computed per direction (FP32, 150,400 nodes; FP64 form 40
 // against 67).  Bound by the latency of one entry's chain.
 // The counter: the deviation forms count the populations that the certified
 // test does not settle (the nodes of zero mesh velocity among them), the FP64
